@@ -18,8 +18,20 @@
 //                   kr (register-resident, one shared-memory exchange), times
 //                   w_{n_t}^{c k1}.
 //   k_pair_filter:  row pairs (k1, R - k1): C-point row FFTs, the pair filter in
-//                   registers (each thread against the elements of one partner
-//                   thread), the inverse row FFTs and the conjugate twiddle.
+//                   registers, the inverse row FFTs and the conjugate twiddle.
+//
+// Storage rule of the spectrum between the passes.  With v[kr] the column transform,
+// row k1 < R / 2 holds v[k1] w_{n_t}^{c k1} and row R - k1 (k1 = 1 .. R / 2) holds
+// conj(v[R - k1]) w_{n_t}^{c k1}.  The same C-point FFT over c of the two rows then
+// gives Z(k) and conj Z(n_t - k) at the same position, k = k1 + R pos:
+// sum_c conj(v[R - k1]) w_{n_t}^{c k1} w_C^{c pos} = conj sum_c v[R - k1] w_{n_t}^{-c k}.
+// So one thread holds both members of every bin pair: no exchange with a partner, one
+// weight evaluation and one stage twiddle for the two, and the sums of both rows are
+// packed instructions.  With (A, B) = (Z(k), conj Z(n_t - k)) the filter is
+// (A, B) <- (a A + b B, a B + b A), and the inverse row FFT and twiddle are again the
+// same for both; the last pass conjugates the rows from R / 2 up.  Rows 0 and R / 2
+// pair with themselves: B = conj A, and A = conj(B) w_C^c.
+//
 //   k_pair_inv_bin: inverse column FFTs into a padded tile; each lane then takes 8
 //                   consecutive samples of a row and bins them for each detector
 //                   with a run accumulator (one vector FP32 reduction per run into
@@ -47,9 +59,6 @@ namespace cmm {
 #endif
 #ifndef CMM_PAIR_XOR
 #define CMM_PAIR_XOR 1     // pixel staging: 0 = rows padded to J + 8 ints, 1 = XOR-swizzled 16-byte chunks (no pad)
-#endif
-#ifndef CMM_PAIR_FILTER_THREADS_PER_SM
-#define CMM_PAIR_FILTER_THREADS_PER_SM 1024
 #endif
 
 // A binning run in the frame of the scan rotation: for samples of one detector on
@@ -148,23 +157,36 @@ __global__ void __launch_bounds__(ColShape<R>::THREADS, ColShape<R>::MINB) k_pai
     x[e] = make_float2(v1, two ? v2 : 0.f);
   }
   ColPlan<R>::template run<-1>(x, i, tw + a.twl.R_off, ad);
-  // four-step twiddle w_N^(c kr), kr = i + e TPC, by recurrence over e
-  float2 w = tw_N(a, tw, c * i);
+  // four-step twiddle w_N^(c k1) by recurrence, k1 = kr for kr = i + e TPC < R / 2 and
+  // k1 = R - kr, the value conjugated, above (see the storage rule at the top)
   const float2 step = tw_N(a, tw, c * TPC);
+  float2 w = tw_N(a, tw, c * i);
   S* Y = reinterpret_cast<S*>(a.spec) + (size_t)q * a.N + c + i * a.C;
 #pragma unroll
-  for (int e = 0; e < kE; ++e) {
+  for (int e = 0; e < kE / 2; ++e) {
     Store<float, S>::st(Y + e * (TPC * a.C), cmul(x[e], w));
+    w = cmul(w, step);
+  }
+  w = tw_N(a, tw, c * (TPC - i));
+#pragma unroll
+  for (int e = kE - 1; e >= kE / 2; --e) {
+    Store<float, S>::st(Y + e * (TPC * a.C), cmulc(w, x[e]));
     w = cmul(w, step);
   }
 }
 
 // ------------------------------------------------------------------ pass F (filter)
+// Both rows of a pair in one thread (2 x 16 complex values): 118 registers, 16 resident
+// warps per SM, 95M warp instructions on 64 detectors x 2^20 samples where one row a
+// thread (32 warps, the partner's values through shared memory) took 151M; 2.85 -> 2.44
+// ms at 1024 x 2^20.  It is now bound by latency (issue 48 %, FP32 pipe 55 % active,
+// DRAM 37 %): 24 warps at 80 registers spill (2.99 ms).  Rows shorter than 128 threads
+// share a CTA of 128 (64: the same times; 256: 85 against 74 us at 128 x 2^18).
 template <int C, int E> struct PairFilterShape {
-  static constexpr int TPR = C / E;
-  static constexpr int THREADS = 2 * TPR > 256 ? 2 * TPR : 256;
-  static constexpr int ROWS = THREADS / TPR;
-  static constexpr int MINB = THREADS >= CMM_PAIR_FILTER_THREADS_PER_SM ? 1 : CMM_PAIR_FILTER_THREADS_PER_SM / THREADS;
+  static constexpr int TPR = C / E;   // threads per row pair
+  static constexpr int THREADS = TPR > 128 ? TPR : 128;
+  static constexpr int PAIRS = THREADS / TPR;   // row pairs per CTA
+  static constexpr int MINB = 512 / THREADS;
 };
 
 template <typename S, int E, int... RC>
@@ -173,73 +195,69 @@ __global__ void __launch_bounds__(PairFilterShape<RadProd<RC...>::value, E>::THR
     k_pair_filter(const TodArgs a, int nd) {
   constexpr int C = RadProd<RC...>::value;
   constexpr int TPR = C / E;
-  constexpr int ROWS = PairFilterShape<C, E>::ROWS;
-  constexpr int PAIRS = ROWS / 2;
+  constexpr int PAIRS = PairFilterShape<C, E>::PAIRS;
   constexpr int PS = clog2(E);
   constexpr int ROWLEN = C + (C >> PS);
-  static_assert(ROWS >= 2 && ROWS % 2 == 0, "a CTA holds whole row pairs");
   if (a.done && *a.done) return;
   extern __shared__ __align__(16) float2 smf[];
   const int rs = threadIdx.x / TPR;
   const int i = threadIdx.x % TPR;
-  const int ps = rs >> 1, side = rs & 1;
-  const int pr = blockIdx.x * PAIRS + ps;
-  const bool pair_ok = pr <= (a.R >> 1);
-  const int ra = pr;
-  const int rb = (a.R - pr) & (a.R - 1);
-  const bool single = ra == rb;
-  const bool active = pair_ok && !(single && side);
-  const int row = side ? rb : ra;
+  const int k1 = blockIdx.x * PAIRS + rs;
+  const bool ok = k1 <= (a.R >> 1);
+  const bool lo = k1 == 0, mid = k1 == (a.R >> 1);   // rows paired with themselves
   const int q = blockIdx.y;
   const bool two = 2 * q + 1 < nd;
   const int d1 = a.d0 + 2 * q, d2 = two ? d1 + 1 : d1;
   const float2* tw = reinterpret_cast<const float2*>(a.tw);
-  S* Y = reinterpret_cast<S*>(a.spec) + (size_t)q * a.N;
-  const RowAddr<PS> ad{smf + rs * ROWLEN};
-  float2 x[E];
-  const int bi = ad.base(i);
+  S* Ya = reinterpret_cast<S*>(a.spec) + (size_t)q * a.N + k1 * C + i;
+  S* Yb = lo ? Ya : Ya + (a.R - 2 * k1) * C;   // row R - k1
+  const RowAddr2<float, PS> ad{reinterpret_cast<Cx2<float>*>(smf) + rs * ROWLEN};
+  Cx2<float> x[E];
 #pragma unroll
-  for (int e = 0; e < E; ++e)
-    x[e] = active ? Store<float, S>::ld(Y + row * C + i + e * TPR) : make_float2(0.f, 0.f);
-  rfft<-1, E, RC...>(x, i, tw + a.twl.C_off, ad);
-  __syncthreads();
+  for (int e = 0; e < E; ++e) {
+    const float2 A = ok ? Store<float, S>::ld(Ya + e * TPR) : make_float2(0.f, 0.f);
+    const float2 B = ok ? Store<float, S>::ld(Yb + e * TPR) : make_float2(0.f, 0.f);
+    x[e] = Cx2<float>{make_float2(A.x, B.x), make_float2(A.y, B.y)};
+  }
+  if (lo) {
 #pragma unroll
-  for (int e = 0; e < E; ++e) ad.st_at(bi, e * TPR, x[e]);
-  const bool wrap = row == 0;
-  const int n = (int)a.N;
-  __syncthreads();
-  // Each thread filters its own elements in registers.  Position pos of row `row`
-  // holds Z(k), k = row + R pos; Z(n - k) sits at position C - 1 - pos of row
-  // R - row (for row 0: (C - pos) mod C of row 0), held by one partner thread;
-  // both threads form a Z + b conj(partner) with the same (a, b), since
-  // min(k, n - k) is the same for the two.  The inverse FFT's first stage starts
-  // with a barrier, so the partner reads below finish before the buffer is reused.
-  if (active) {
-    const float4 cf1 = reinterpret_cast<const float4*>(a.coef)[d1];
-    const float4 cf2 = reinterpret_cast<const float4*>(a.coef)[d2];
-    const RowAddr<PS> pa{smf + (single ? rs : (rs ^ 1)) * ROWLEN};
+    for (int e = 0; e < E; ++e) x[e].im.y = -x[e].im.x;   // B = conj A
+  } else if (mid) {
+    // row R / 2 is stored as B = conj(y) w_N^(c R / 2): A = conj(B) w_C^c
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-      const int pos = i + e * TPR;
-      const int pp = wrap ? ((C - pos) & (C - 1)) : (C - 1 - pos);
-      const float2 B = pa.ld(pp);
-      const int k = row + a.R * pos;
-      const int kf = min(k, n - k);
+      const float2 A = cmul(make_float2(x[e].re.y, -x[e].im.y), __ldg(tw + a.twl.C_off + i + e * TPR));
+      x[e].re.x = A.x;
+      x[e].im.x = A.y;
+    }
+  }
+  rfft2<float, -1, true, E, RC...>(x, i, tw + a.twl.C_off, ad);
+  {
+    const float4 cf1 = reinterpret_cast<const float4*>(a.coef)[d1];
+    const float4 cf2 = reinterpret_cast<const float4*>(a.coef)[d2];
+    const int n = (int)a.N;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int k = k1 + a.R * (i + e * TPR);
+      const int kf = ok ? min(k, n - k) : 0;
       float w1, w2;
       pair_weights(a, d1, d2, cf1, cf2, two, kf, w1, w2);
       const float ha = 0.5f * (w1 + w2), hb = 0.5f * (w1 - w2);
-      x[e] = make_float2(fmaf(ha, x[e].x, hb * B.x), fmaf(ha, x[e].y, -hb * B.y));
+      const float2 h{ha, ha}, g{hb, hb};
+      x[e].re = pfma(h, x[e].re, pmul(g, make_float2(x[e].re.y, x[e].re.x)));
+      x[e].im = pfma(h, x[e].im, pmul(g, make_float2(x[e].im.y, x[e].im.x)));
     }
   }
-  rfft<1, E, RC...>(x, i, tw + a.twl.C_off, ad);
-  if (active) {
-    // w_N^(row c), c = i + e TPR, by recurrence over e
-    float2 w = tw_N(a, tw, row * i);
-    const float2 stp = tw_N(a, tw, row * TPR);
-    S* Yr = Y + row * C + i;
+  rfft2<float, 1, false, E, RC...>(x, i, tw + a.twl.C_off, ad);
+  if (ok) {
+    // conj(w_N^(k1 c)), c = i + e TPR, by recurrence over e, for both rows
+    float2 w = tw_N(a, tw, k1 * i);
+    const float2 stp = tw_N(a, tw, k1 * TPR);
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-      Store<float, S>::st(Yr + e * TPR, cmulc(x[e], w));
+      const Cx2<float> y = cx_mul<float>(x[e], w.x, -w.y);
+      if (!mid) Store<float, S>::st(Ya + e * TPR, make_float2(y.re.x, y.im.x));
+      if (!lo) Store<float, S>::st(Yb + e * TPR, make_float2(y.re.y, y.im.y));
       w = cmul(w, stp);
     }
   }
@@ -279,7 +297,10 @@ __global__ void __launch_bounds__(ColShape<R>::THREADS, ColShape<R>::MINB_INV) k
   const S* Y = reinterpret_cast<const S*>(a.spec) + (size_t)q * a.N + c + i * a.C;
   float2 x[kE];
 #pragma unroll
-  for (int e = 0; e < kE; ++e) x[e] = Store<float, S>::ld(Y + e * (TPC * a.C));
+  for (int e = 0; e < kE; ++e) {
+    x[e] = Store<float, S>::ld(Y + e * (TPC * a.C));
+    if (e >= kE / 2) x[e].y = -x[e].y;   // rows R / 2 and above are stored conjugated
+  }
   ColPlan<R>::template run<1>(x, i, tw + a.twl.R_off, ad);
   __syncthreads();
   // y(t) for t = c + C kr into a tile of rows kr
@@ -472,10 +493,9 @@ static int dispatch_pair_T(const TodArgs& a, int nd, int pass, cudaStream_t st, 
 template <typename S, int E, int... RC>
 static int run_pair_F(const TodArgs& a, int nd, cudaStream_t st, bool attr_only) {
   constexpr int C = RadProd<RC...>::value;
-  constexpr int ROWS = PairFilterShape<C, E>::ROWS;
-  constexpr int PAIRS = ROWS / 2;
+  constexpr int PAIRS = PairFilterShape<C, E>::PAIRS;
   constexpr int PS = clog2(E);
-  const size_t smem = sizeof(float2) * ROWS * (C + (C >> PS));
+  const size_t smem = sizeof(Cx2<float>) * PAIRS * (C + (C >> PS));
   if (attr_only) {
     CMM_CUDA(cudaFuncSetAttribute(k_pair_filter<S, E, RC...>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     return CMM_OK;
