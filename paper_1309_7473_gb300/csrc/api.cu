@@ -271,7 +271,7 @@ int cmm_pointing_create(cmm_ctx* ctx, const cmm_map_geom* geom, int32_t n_det, c
     k_rot2<<<(int)std::min<long long>((n_samp + 255) / 256, 4096), 256, 0, st>>>(pt->bore, n_samp, pt->rot2);
     CMM_LAUNCH_CHECK();
     CMM_CUDA(cudaMemsetAsync(blocks, 0, sizeof(double) * nb * pt->npix, st));
-    CMM_TRY(launch_hit_blocks(pt, nullptr, nullptr, blocks, nullptr));
+    CMM_TRY(launch_hit_blocks(pt, nullptr, nullptr, blocks));
     CMM_TRY(launch_mask_from_hits(pt, blocks));
     CMM_CUDA(cudaStreamSynchronize(st));
     return CMM_OK;
@@ -911,7 +911,7 @@ static int circulant_build(cmm_precon* pc, const cmm_precon_opts* o) {
     CMM_TRY(dalloc(&pc->tmp, sizeof(double) * nc * npix));
     // Eq. 7: Sigma^T Sigma = binned blocks
     CMM_CUDA(cudaMemsetAsync(blocks, 0, sizeof(double) * nb * npix, st));
-    CMM_TRY(launch_hit_blocks(pt, precon_weights(op, o), pt->mask, blocks, nullptr));
+    CMM_TRY(launch_hit_blocks(pt, precon_weights(op, o), pt->mask, blocks));
     CMM_TRY(launch_block_sqrt(nc, npix, blocks, pt->mask, pc->sig, pc->sig_inv, st));
     // reference pixel
     std::vector<uint8_t> mask(npix);
@@ -933,7 +933,7 @@ static int circulant_build(cmm_precon* pc, const cmm_precon_opts* o) {
     CMM_TRY(launch_circ_q<double>(nc, rows, pc->sig_inv, (int)ref, pt->ny, pt->nx, taper, qplanes, st));
     CMM_TRY(fft2<double>(plan64, qplanes, nc * nc, -1, nullptr, st));
     const double eps = (o && o->pd_eps > 0) ? o->pd_eps : 1e-6;
-    CMM_TRY(launch_mode_inverse<double>(nc, qplanes, npix, eps, pc->hinv, scratch, st));
+    CMM_TRY(launch_mode_inverse(nc, qplanes, pt->ny, pt->nx, eps, pc->hinv, scratch, st));
     if (op->prec != CMM_PREC_F64) {
       // the apply of an FP32 operator multiplies FP32 spectra: FP32 blocks (GB300's
       // FP64 pipe would otherwise bound the per-mode products)
@@ -946,7 +946,7 @@ static int circulant_build(cmm_precon* pc, const cmm_precon_opts* o) {
     unsigned long long h[2];
     CMM_CUDA(cudaMemcpyAsync(h, scratch, sizeof(h), cudaMemcpyDeviceToHost, st));
     CMM_CUDA(cudaStreamSynchronize(st));
-    pc->n_clamped = (int64_t)(h[1] / 2);
+    pc->n_clamped = (int64_t)h[1];
     return CMM_OK;
   };
   int s = run();
@@ -981,7 +981,7 @@ int cmm_precon_create(cmm_op* op, int32_t kind, const cmm_precon_opts* opts, cmm
       auto run = [&]() -> int {
         CMM_CUDA(cudaMemsetAsync(blocks, 0, sizeof(double) * nb * pt->npix, st));
         CMM_TRY(launch_hit_blocks(pt, kind == CMM_PRECON_BINNED ? precon_weights(op, opts) : nullptr, pt->mask,
-                                  blocks, nullptr));
+                                  blocks));
         CMM_TRY(launch_block_inverse(pt->ncomp, pt->npix, blocks, pt->mask, pc->inv, st));
         CMM_CUDA(cudaStreamSynchronize(st));
         return CMM_OK;

@@ -214,8 +214,7 @@ int launch_map_to_gather(cmm_op* op, const double* m);
 int launch_acc_to_map(cmm_op* op, double* out);
 int launch_apply_chunk(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, int pass = -1);
 int launch_project(cmm_op* op, const double* m, void* tod, int tod_is_f64);
-int launch_hit_blocks(cmm_pointing* pt, const double* det_weight, const uint8_t* mask,
-                      double* blocks, const int* done);
+int launch_hit_blocks(cmm_pointing* pt, const double* det_weight, const uint8_t* mask, double* blocks);
 int op_init_twiddles(cmm_op* op);
 int op_prepare_kernels(cmm_op* op);
 int launch_fill_pixels(cmm_op* op);

@@ -97,8 +97,7 @@ template <typename T> int fft2(const Fft2Plan& p, V2<T>* data, int nplanes, int 
 template <typename T>
 int launch_circ_q(int ncomp, const double* rows, const double* sig_inv, int ref, int ny, int nx,
                   double taper_sigma, V2<T>* planes, cudaStream_t s);
-template <typename T>
-int launch_mode_inverse(int ncomp, const V2<T>* planes, long long npix, double eps, double* hinv,
+int launch_mode_inverse(int ncomp, const double2* planes, int ny, int nx, double eps, double* hinv,
                         unsigned long long* scratch2, cudaStream_t s);
 template <typename T>
 int launch_real_to_planes(const double* x, V2<T>* planes, long long n, const int* done, cudaStream_t s);
