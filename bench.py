@@ -456,7 +456,8 @@ def run_ours(args, rank, world):
         "setup_seconds": round(setup_s, 2),
         "clocks": clocks,
     }
-    out["gpu_launches"] = launches_per_iteration(scan.n_det, chunk_dets) * args.steps + SETUP_LAUNCHES + CIRC_LAUNCHES
+    out["gpu_launches"] = (launches_per_iteration(scan.n_det, chunk_dets, CIRC_FUSED_LAUNCHES) * args.steps
+                           + SETUP_LAUNCHES + CIRC_FUSED_LAUNCHES)
     return out
 
 
@@ -652,18 +653,19 @@ def cufft_filter_ms(scan, noise, dev, stream):
                     "excludes P and P^T", "ms": ms}
 
 
-def launches_per_iteration(n_det, chunk):
+def launches_per_iteration(n_det, chunk, circ=None):
     """Kernels of one circulant-PCG iteration: the A-application (map copy in, per
     chunk one forward and one filter launch and, per 2048 detectors (eight FP32
     partial maps of 256 detectors), one inverse + binning launch and one flush; map
-    copy out), the CG update kernels and the circulant preconditioner (Sigma^-1,
+    copy out), the CG update kernels and the circulant preconditioner: `circ`
+    kernels, by default those of the maps that the line FFTs serve (Sigma^-1,
     2-D FFTs, per-mode solve)."""
     a = 2
     maps = min(8, max(1, math.ceil(chunk / 256)))
     for d0 in range(0, n_det, chunk):
         nd = min(chunk, n_det - d0)
         a += 2 + 2 * math.ceil(nd / (256 * maps))
-    return a + CG_LAUNCHES + CIRC_LAUNCHES
+    return a + CG_LAUNCHES + (CIRC_LAUNCHES if circ is None else circ)
 
 
 # kernels per iteration outside the A-application (cmm_solve's FP64 PCG step):
@@ -672,8 +674,11 @@ CG_LAUNCHES = 6
 # the circulant apply: Sigma^-1 into the packed planes, 2 + 2 line-FFT passes, the
 # per-mode products, Sigma^-1 out of the planes with the r^T z partials
 CIRC_LAUNCHES = 7
+# the same on TQU maps whose sides fit the fused kernels (1200 x 900 among them): rows
+# with Sigma^-1, columns with the per-mode products, rows with Sigma^-1 and r^T z
+CIRC_FUSED_LAUNCHES = 3
 # once per cmm_solve call before its iterations: b^T b (partials and sum), r0, the
-# solver state (plus one preconditioner apply, CIRC_LAUNCHES)
+# solver state (plus one preconditioner apply)
 SETUP_LAUNCHES = 4
 
 

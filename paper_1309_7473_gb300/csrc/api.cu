@@ -10,6 +10,7 @@
 #include <string>
 #include <vector>
 
+#include "circ.cuh"
 #include "common.cuh"
 #include "map_kernels.cuh"
 
@@ -124,14 +125,13 @@ struct cmm_precon {
   cmm_op* op = nullptr;
   int kind = 0;
   double* inv = nullptr;       // binned / Jacobi: inverse blocks
-  double* sig = nullptr;       // circulant: Sigma
   double* sig_inv = nullptr;   // circulant: Sigma^-1
   float* sig_inv32 = nullptr;  // its FP32 copy, for the apply of FP32/BF16 operators
   double* hinv = nullptr;      // circulant: per-mode packed inverse
   float* hinv32 = nullptr;     // its FP32 copy, applied with the FP32 map FFTs of FP32/BF16 operators
-  void* planes = nullptr;      // complex workspace [ncomp][npix]
-  double* tmp = nullptr;       // [ncomp * npix]
+  void* planes = nullptr;      // complex workspace [ncomp][npix] (fused apply: one Cx2 per pixel)
   Fft2Plan plan;
+  CircPlan fused;              // TQU maps whose sides the fused kernels take (circ.cu)
   int64_t n_clamped = 0;
   int64_t ref = -1;
   double taper = 0.0;
@@ -760,13 +760,11 @@ int cmm_precon_destroy(cmm_precon* pc) {
   cudaSetDevice(pc->op->ctx->device);
   cudaStreamSynchronize(pc->op->ctx->stream);
   dfree(pc->inv);
-  dfree(pc->sig);
   dfree(pc->sig_inv);
   dfree(pc->sig_inv32);
   dfree(pc->hinv);
   dfree(pc->hinv32);
   dfree(pc->planes);
-  dfree(pc->tmp);
   dfree(pc->plan.tw);
   dfree(pc->sqrt_phi);
   dfree(pc->ttmp);
@@ -883,6 +881,11 @@ static int circulant_build(cmm_precon* pc, const cmm_precon_opts* o) {
   const int64_t npix = pt->npix;
   const int nb = nc == 1 ? 1 : 6;
   CMM_TRY(fft2_plan_init<T>(pc->plan, pt->ny, pt->nx));
+  if (nc == 3) {
+    pc->fused = circ_plan<T>(pt->ny, pt->nx);
+    if (pc->fused.ok) CMM_TRY(circ_prepare<T>(pc->fused));
+  }
+  const int64_t n_hinv = nc == 1 ? npix : 9 * (pc->fused.ok ? pc->fused.modes() : npix);
   // the build (q, its transform and the per-mode inverse) is FP64 in every precision
   // mode; only the apply's transforms follow the operator's precision
   Fft2Plan plan64;
@@ -904,15 +907,13 @@ static int circulant_build(cmm_precon* pc, const cmm_precon_opts* o) {
     CMM_TRY(dalloc(&rows, sizeof(double) * nc * nc * npix));
     CMM_TRY(dalloc(&qplanes, sizeof(double2) * nc * nc * npix));
     CMM_TRY(dalloc(&scratch, sizeof(unsigned long long) * 2));
-    CMM_TRY(dalloc(&pc->sig, sizeof(double) * nb * npix));
     CMM_TRY(dalloc(&pc->sig_inv, sizeof(double) * nb * npix));
-    CMM_TRY(dalloc(&pc->hinv, sizeof(double) * (nc == 1 ? 1 : 9) * npix));
-    CMM_TRY(dalloc(&pc->planes, sizeof(V2<T>) * nc * npix));
-    CMM_TRY(dalloc(&pc->tmp, sizeof(double) * nc * npix));
+    CMM_TRY(dalloc(&pc->hinv, sizeof(double) * n_hinv));
+    CMM_TRY(dalloc(&pc->planes, sizeof(V2<T>) * (pc->fused.ok ? 2 : nc) * npix));
     // Eq. 7: Sigma^T Sigma = binned blocks
     CMM_CUDA(cudaMemsetAsync(blocks, 0, sizeof(double) * nb * npix, st));
     CMM_TRY(launch_hit_blocks(pt, precon_weights(op, o), pt->mask, blocks));
-    CMM_TRY(launch_block_sqrt(nc, npix, blocks, pt->mask, pc->sig, pc->sig_inv, st));
+    CMM_TRY(launch_block_sqrt(nc, npix, blocks, pt->mask, pc->sig_inv, st));
     // reference pixel
     std::vector<uint8_t> mask(npix);
     CMM_CUDA(cudaMemcpyAsync(mask.data(), pt->mask, npix, cudaMemcpyDeviceToHost, st));
@@ -933,13 +934,12 @@ static int circulant_build(cmm_precon* pc, const cmm_precon_opts* o) {
     CMM_TRY(launch_circ_q<double>(nc, rows, pc->sig_inv, (int)ref, pt->ny, pt->nx, taper, qplanes, st));
     CMM_TRY(fft2<double>(plan64, qplanes, nc * nc, -1, nullptr, st));
     const double eps = (o && o->pd_eps > 0) ? o->pd_eps : 1e-6;
-    CMM_TRY(launch_mode_inverse(nc, qplanes, pt->ny, pt->nx, eps, pc->hinv, scratch, st));
+    CMM_TRY(launch_mode_inverse(nc, qplanes, pt->ny, pt->nx, eps, pc->hinv, pc->fused.ok ? pc->fused.J : 0, scratch, st));
     if (op->prec != CMM_PREC_F64) {
       // the apply of an FP32 operator multiplies FP32 spectra: FP32 blocks (GB300's
       // FP64 pipe would otherwise bound the per-mode products)
-      const int64_t nh = (int64_t)(nc == 1 ? 1 : 9) * npix;
-      CMM_TRY(dalloc(&pc->hinv32, sizeof(float) * nh));
-      CMM_TRY(launch_to_f32(pc->hinv, pc->hinv32, nh, st));
+      CMM_TRY(dalloc(&pc->hinv32, sizeof(float) * n_hinv));
+      CMM_TRY(launch_to_f32(pc->hinv, pc->hinv32, n_hinv, st));
       CMM_TRY(dalloc(&pc->sig_inv32, sizeof(float) * nb * npix));
       CMM_TRY(launch_to_f32(pc->sig_inv, pc->sig_inv32, nb * npix, st));
     }
@@ -1016,6 +1016,13 @@ static int circulant_apply(cmm_precon* pc, const double* r, double* z, double* p
   // moves into and out of the complex planes; TQU maps travel as two complex planes
   // (T + i Q and U), so three real transforms take two complex ones
   if (nc == 3) {
+    if (pc->fused.ok) {
+      const V2<T>* tw = (const V2<T>*)pc->plan.tw;
+      if constexpr (sizeof(T) == 4)
+        return launch_circ_apply<T>(pc->fused, tw, pc->sig_inv32, pc->hinv32, r, z, planes, partial, done, st);
+      else
+        return launch_circ_apply<T>(pc->fused, tw, pc->sig_inv, pc->hinv, r, z, planes, partial, done, st);
+    }
     if constexpr (sizeof(T) == 4) {
       if (pc->hinv32 && pc->sig_inv32) {
         // FP32 operator: Sigma^-1 and the mode blocks in FP32 (FP64 build, FP32 copies)

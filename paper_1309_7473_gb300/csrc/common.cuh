@@ -244,8 +244,8 @@ bool unet_matches(const cmm_unet* u, const cmm_ctx* ctx, int ny, int nx);
 int launch_mask_from_hits(cmm_pointing* pt, const double* blocks);
 int launch_block_inverse(int ncomp, int64_t npix, const double* blocks, const uint8_t* mask,
                          double* inv, cudaStream_t s);
-int launch_block_sqrt(int ncomp, int64_t npix, const double* blocks, const uint8_t* mask,
-                      double* sig, double* sig_inv, cudaStream_t s);
+int launch_block_sqrt(int ncomp, int64_t npix, const double* blocks, const uint8_t* mask, double* sig_inv,
+                      cudaStream_t s);
 int launch_block_apply(int ncomp, int64_t npix, const double* blocks, const double* x,
                        double* y, const int* done, cudaStream_t s);
 int launch_dot(const double* x, const double* y, int64_t n, double* partial, double* out,

@@ -119,7 +119,7 @@ struct RowAddr {
 // part, a product by i is a renaming, and a stage twiddle serves both (one
 // recurrence for two sequences).
 template <typename T>
-struct Cx2 {
+struct __align__(16) Cx2 {
   V2<T> re, im;
 };
 

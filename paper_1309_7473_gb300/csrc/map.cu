@@ -141,44 +141,33 @@ __global__ void k_block_inverse(const double* __restrict__ blocks, const uint8_t
   }
 }
 
-// Sigma = B^(1/2), Sigma^-1 = B^(-1/2) (symmetric) per unmasked pixel.
+// Sigma^-1 = B^(-1/2) (symmetric) per unmasked pixel.
 template <int NC>
 __global__ void k_block_sqrt(const double* __restrict__ blocks, const uint8_t* __restrict__ mask,
-                             double* __restrict__ sig, double* __restrict__ sig_inv, long long npix) {
+                             double* __restrict__ sig_inv, long long npix) {
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < npix;
        p += (long long)gridDim.x * blockDim.x) {
     if (NC == 1) {
-      const double b = blocks[p];
-      sig[p] = mask[p] ? sqrt(b) : 0.0;
-      sig_inv[p] = mask[p] ? 1.0 / sqrt(b) : 0.0;
+      sig_inv[p] = mask[p] ? 1.0 / sqrt(blocks[p]) : 0.0;
       continue;
     }
-    double* s = sig + 6 * p;
     double* si = sig_inv + 6 * p;
     if (!mask[p]) {
-      for (int i = 0; i < 6; ++i) s[i] = si[i] = 0.0;
+      for (int i = 0; i < 6; ++i) si[i] = 0.0;
       continue;
     }
     double a[3][3], v[3][3];
     sym3_load(blocks + 6 * p, a);
     jacobi_eigen<3>(a, v);
-    double r[3], ri[3];
-    for (int k = 0; k < 3; ++k) {
-      r[k] = sqrt(a[k][k]);
-      ri[k] = 1.0 / r[k];
-    }
-    double m[3][3], mi[3][3];
+    double ri[3];
+    for (int k = 0; k < 3; ++k) ri[k] = 1.0 / sqrt(a[k][k]);
+    double mi[3][3];
     for (int i = 0; i < 3; ++i)
       for (int j = 0; j < 3; ++j) {
-        double x = 0, y = 0;
-        for (int k = 0; k < 3; ++k) {
-          x += v[i][k] * r[k] * v[j][k];
-          y += v[i][k] * ri[k] * v[j][k];
-        }
-        m[i][j] = x;
+        double y = 0;
+        for (int k = 0; k < 3; ++k) y += v[i][k] * ri[k] * v[j][k];
         mi[i][j] = y;
       }
-    sym3_store(s, m);
     sym3_store(si, mi);
   }
 }
@@ -735,16 +724,21 @@ __global__ void k_mode_maxeig(const double2* __restrict__ planes, int ny, int nx
   if ((threadIdx.x & 31) == 0 && local > 0.0) atomicMax(maxbits, (unsigned long long)__double_as_longlong(local));
 }
 
+// J = 0: hinv [npix][9] in mode order, both members of a mirror pair; J > 0: the half
+// kx <= nx / 2 in the order of k_circ_cols, [kx / J][ky][kx % J][9].
 template <int NC>
 __global__ void k_mode_inverse(const double2* __restrict__ planes, int ny, int nx,
                                const unsigned long long* __restrict__ maxbits, double eps,
-                               double* __restrict__ hinv, unsigned long long* __restrict__ nclamp) {
+                               double* __restrict__ hinv, int J, unsigned long long* __restrict__ nclamp) {
   const long long npix = (long long)ny * nx;
   const double floor_ = eps * __longlong_as_double((long long)*maxbits);
   for (long long f = blockIdx.x * (long long)blockDim.x + threadIdx.x; f < npix;
        f += (long long)gridDim.x * blockDim.x) {
     const long long g = mirror_mode(f, ny, nx);
-    if (g < f) continue;
+    const int ky = (int)(f / nx), kx = (int)(f - (long long)ky * nx);
+    // the member of the pair that this thread serves, and whether it counts for both
+    if (J > 0 ? kx > nx / 2 : g < f) continue;
+    const bool both = J > 0 ? !(kx == 0 || 2 * kx == nx) : g != f;
     int nc = 0;
     if (NC == 1) {
       const double h = planes[f].x;
@@ -770,12 +764,13 @@ __global__ void k_mode_inverse(const double2* __restrict__ planes, int ny, int n
       } else {
         nc = herm3_floored_inverse(h, floor_, o);
       }
+      const long long at = J > 0 ? ((long long)(kx / J) * ny + ky) * J + kx % J : f;
       for (int j = 0; j < 9; ++j) {
-        hinv[9 * f + j] = o[j];
-        if (g != f) hinv[9 * g + j] = (j == 4 || j == 6 || j == 8) ? -o[j] : o[j];
+        hinv[9 * at + j] = o[j];
+        if (J == 0 && g != f) hinv[9 * g + j] = (j == 4 || j == 6 || j == 8) ? -o[j] : o[j];
       }
     }
-    if (nc) atomicAdd(nclamp, (unsigned long long)(g != f ? 2 * nc : nc));
+    if (nc) atomicAdd(nclamp, (unsigned long long)(both ? 2 * nc : nc));
   }
 }
 
@@ -892,19 +887,6 @@ __global__ void k_planes_block_dot_packed(const V2<T>* __restrict__ planes, doub
     if (w) acc += w[p] * y0 + w[npix + p] * y1 + w[2 * npix + p] * y2;
   }
   if (partial) block_sum_store(acc, partial);
-}
-
-// Y = H^-1 X for one mode from its packed Hermitian block (d0 d1 d2, h01 h02 h12)
-template <typename H>
-__device__ __forceinline__ void mode_mul3(const H* __restrict__ o, const H (&xr)[3], const H (&xi)[3], H (&yr)[3],
-                                          H (&yi)[3]) {
-  const H h01r = o[3], h01i = o[4], h02r = o[5], h02i = o[6], h12r = o[7], h12i = o[8];
-  yr[0] = o[0] * xr[0] + (h01r * xr[1] - h01i * xi[1]) + (h02r * xr[2] - h02i * xi[2]);
-  yi[0] = o[0] * xi[0] + (h01r * xi[1] + h01i * xr[1]) + (h02r * xi[2] + h02i * xr[2]);
-  yr[1] = (h01r * xr[0] + h01i * xi[0]) + o[1] * xr[1] + (h12r * xr[2] - h12i * xi[2]);
-  yi[1] = (h01r * xi[0] - h01i * xr[0]) + o[1] * xi[1] + (h12r * xi[2] + h12i * xr[2]);
-  yr[2] = (h02r * xr[0] + h02i * xi[0]) + (h12r * xr[1] + h12i * xi[1]) + o[2] * xr[2];
-  yi[2] = (h02r * xi[0] - h02i * xr[0]) + (h12r * xi[1] - h12i * xr[1]) + o[2] * xi[2];
 }
 
 // The per-mode products on the packed spectra: each thread takes a mode f and its
@@ -1057,10 +1039,10 @@ int launch_block_inverse(int ncomp, int64_t npix, const double* blocks, const ui
   return CMM_OK;
 }
 
-int launch_block_sqrt(int ncomp, int64_t npix, const double* blocks, const uint8_t* mask, double* sig,
-                      double* sig_inv, cudaStream_t s) {
-  if (ncomp == 1) k_block_sqrt<1><<<grid_for(npix), 256, 0, s>>>(blocks, mask, sig, sig_inv, npix);
-  else k_block_sqrt<3><<<grid_for(npix), 256, 0, s>>>(blocks, mask, sig, sig_inv, npix);
+int launch_block_sqrt(int ncomp, int64_t npix, const double* blocks, const uint8_t* mask, double* sig_inv,
+                      cudaStream_t s) {
+  if (ncomp == 1) k_block_sqrt<1><<<grid_for(npix), 256, 0, s>>>(blocks, mask, sig_inv, npix);
+  else k_block_sqrt<3><<<grid_for(npix), 256, 0, s>>>(blocks, mask, sig_inv, npix);
   CMM_LAUNCH_CHECK();
   return CMM_OK;
 }
@@ -1302,16 +1284,16 @@ int launch_circ_q(int ncomp, const double* rows, const double* sig_inv, int ref,
 template int launch_circ_q<float>(int, const double*, const double*, int, int, int, double, float2*, cudaStream_t);
 template int launch_circ_q<double>(int, const double*, const double*, int, int, int, double, double2*, cudaStream_t);
 
-int launch_mode_inverse(int ncomp, const double2* planes, int ny, int nx, double eps, double* hinv,
+int launch_mode_inverse(int ncomp, const double2* planes, int ny, int nx, double eps, double* hinv, int J,
                         unsigned long long* scratch2, cudaStream_t s) {
   CMM_CUDA(cudaMemsetAsync(scratch2, 0, 2 * sizeof(unsigned long long), s));
   const long long npix = (long long)ny * nx;
   if (ncomp == 1) {
     k_mode_maxeig<1><<<grid_for(npix), 256, 0, s>>>(planes, ny, nx, scratch2);
-    k_mode_inverse<1><<<grid_for(npix), 256, 0, s>>>(planes, ny, nx, scratch2, eps, hinv, scratch2 + 1);
+    k_mode_inverse<1><<<grid_for(npix), 256, 0, s>>>(planes, ny, nx, scratch2, eps, hinv, J, scratch2 + 1);
   } else {
     k_mode_maxeig<3><<<grid_for(npix), 128, 0, s>>>(planes, ny, nx, scratch2);
-    k_mode_inverse<3><<<grid_for(npix), 128, 0, s>>>(planes, ny, nx, scratch2, eps, hinv, scratch2 + 1);
+    k_mode_inverse<3><<<grid_for(npix), 128, 0, s>>>(planes, ny, nx, scratch2, eps, hinv, J, scratch2 + 1);
   }
   CMM_LAUNCH_CHECK();
   return CMM_OK;

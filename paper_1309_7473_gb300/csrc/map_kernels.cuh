@@ -55,6 +55,19 @@ __device__ __forceinline__ double block_sum_all(const double* partial, int n) {
   return r;
 }
 
+// Y = H^-1 X for one mode from its packed Hermitian block (d0 d1 d2, h01 h02 h12)
+template <typename H>
+__device__ __forceinline__ void mode_mul3(const H* __restrict__ o, const H (&xr)[3], const H (&xi)[3], H (&yr)[3],
+                                          H (&yi)[3]) {
+  const H h01r = o[3], h01i = o[4], h02r = o[5], h02i = o[6], h12r = o[7], h12i = o[8];
+  yr[0] = o[0] * xr[0] + (h01r * xr[1] - h01i * xi[1]) + (h02r * xr[2] - h02i * xi[2]);
+  yi[0] = o[0] * xi[0] + (h01r * xi[1] + h01i * xr[1]) + (h02r * xi[2] + h02i * xr[2]);
+  yr[1] = (h01r * xr[0] + h01i * xi[0]) + o[1] * xr[1] + (h12r * xr[2] - h12i * xi[2]);
+  yi[1] = (h01r * xi[0] - h01i * xr[0]) + o[1] * xi[1] + (h12r * xi[2] + h12i * xr[2]);
+  yr[2] = (h02r * xr[0] + h02i * xi[0]) + (h12r * xr[1] + h12i * xi[1]) + o[2] * xr[2];
+  yi[2] = (h02r * xi[0] - h02i * xr[0]) + (h12r * xi[1] - h12i * xr[1]) + o[2] * xi[2];
+}
+
 int launch_block_apply_dot(int ncomp, int64_t npix, const double* blk, const double* x, double* y,
                            const double* w, double* partial, const int* done, cudaStream_t s);
 // y = d .* x and z = (first ? 0 : z) + d .* x on every Stokes component (d [npix])
@@ -97,7 +110,7 @@ template <typename T> int fft2(const Fft2Plan& p, V2<T>* data, int nplanes, int 
 template <typename T>
 int launch_circ_q(int ncomp, const double* rows, const double* sig_inv, int ref, int ny, int nx,
                   double taper_sigma, V2<T>* planes, cudaStream_t s);
-int launch_mode_inverse(int ncomp, const double2* planes, int ny, int nx, double eps, double* hinv,
+int launch_mode_inverse(int ncomp, const double2* planes, int ny, int nx, double eps, double* hinv, int J,
                         unsigned long long* scratch2, cudaStream_t s);
 template <typename T>
 int launch_real_to_planes(const double* x, V2<T>* planes, long long n, const int* done, cudaStream_t s);
