@@ -395,6 +395,8 @@ static void free_op(cmm_op* op) {
   dfree(op->acc32);
   dfree(op->tw);
   dfree(op->tw_pair);
+  dfree(op->rot64);
+  dfree(op->lg2);
   dfree(op->tmp_a);
   dfree(op->tmp_b);
   dfree(op->pix);
@@ -1502,7 +1504,7 @@ int cmm_autotune(cmm_op* op, int32_t reps, const char* cache_path, int32_t* chos
   CMM_CUDA(cudaSetDevice(op->ctx->device));
   const TuneKey key{op->pt->n_t, op->pt->n_det, op->prec, op->pt->ncomp};
   const int logN = op->logR + op->logC;
-  const bool pair_ok = op->pR > 0 && op->tw_pair && op->nz->corr_r == 0 && op->pt->max_hits <= kF32HitLimit;
+  const bool pair_ok = pair_path_fits(op);
   auto valid = [&](int v) { return (v == 0 && pair_ok) || (v > 0 && v < logN); };
   // cached decision (process-wide, then the optional file)
   for (auto& e : g_tune_cache)
@@ -1534,7 +1536,7 @@ int cmm_autotune(cmm_op* op, int32_t reps, const char* cache_path, int32_t* chos
   if (pair_ok) cand.push_back(0);
   for (int lr = 6; lr <= 8; ++lr)
     if (logN - lr >= 6 && logN - lr <= 12 && op->prec != CMM_PREC_F64) cand.push_back(lr);
-  if (cand.empty()) cand.push_back(op->logR);
+  if (cand.empty() || op->prec == CMM_PREC_F64) cand.push_back(op->logR);   // the generic kernels
   const size_t bytes = sizeof(double) * op->pt->ncomp * op->pt->npix;
   CMM_CUDA(cudaMemsetAsync(op->tmp_a, 0, bytes, op->ctx->stream));
   cudaEvent_t e0, e1;

@@ -87,14 +87,6 @@ __device__ __forceinline__ Cx2<T> cx_scale(T c, const Cx2<T>& a) {
   const V2<T> cc{c, c};
   return Cx2<T>{pmul(cc, a.re), pmul(cc, a.im)};
 }
-// a + SIGN i b and a - SIGN i b
-template <typename T, int SIGN>
-__device__ __forceinline__ void cx_addsub_i(const Cx2<T>& a, const Cx2<T>& b, Cx2<T>& plus, Cx2<T>& minus) {
-  const Cx2<T> p{psub(a.re, b.im), padd(a.im, b.re)}, m{padd(a.re, b.im), psub(a.im, b.re)};
-  plus = SIGN > 0 ? p : m;
-  minus = SIGN > 0 ? m : p;
-}
-
 // x_q <- sum_j x_j exp(SIGN 2 pi i j q / N): direct forms for 2 to 5, N = A B else
 // (A-point transforms, the constants w_N^(b c), B-point transforms)
 template <typename T, int N, int SIGN>
@@ -135,8 +127,7 @@ __device__ __forceinline__ void cx_dft_n(Cx2<T>* x) {
         if constexpr (b * c == 0) {
         } else if constexpr (4 * b * c == N) {   // SIGN i
           const Cx2<T> v = y[b][c];
-          const V2<T> zero{(T)0, (T)0};
-          y[b][c] = SIGN > 0 ? Cx2<T>{psub(zero, v.im), v.re} : Cx2<T>{v.im, psub(zero, v.re)};
+          y[b][c] = SIGN > 0 ? Cx2<T>{V2<T>{-v.im.x, -v.im.y}, v.re} : Cx2<T>{v.im, V2<T>{-v.re.x, -v.re.y}};
         } else {
           y[b][c] = cx_mul<T>(y[b][c], (T)wr, (T)wi);
         }

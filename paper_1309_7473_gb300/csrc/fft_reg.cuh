@@ -30,9 +30,15 @@ template <int... Rs> struct RadProd;
 template <> struct RadProd<> { static constexpr int value = 1; };
 template <int R, int... Rs> struct RadProd<R, Rs...> { static constexpr int value = R * RadProd<Rs...>::value; };
 
-template <int SIGN, int E, int L, int P, typename Addr, int R, int... REST>
-__device__ __forceinline__ void rfft_stages(float2 (&x)[E], const int i, const float2* __restrict__ tw,
-                                            const Addr& ad) {
+// the real type of a complex pair
+template <typename V> struct RealOf;
+template <> struct RealOf<float2> { using t = float; };
+template <> struct RealOf<double2> { using t = double; };
+
+// FP64 takes every stage twiddle from the table: loads cost nothing beside its pipe.
+template <int SIGN, int E, int L, int P, typename V, typename Addr, int R, int... REST>
+__device__ __forceinline__ void rfft_stages(V (&x)[E], const int i, const V* __restrict__ tw, const Addr& ad) {
+  using T = typename RealOf<V>::t;
   static_assert(E % R == 0, "every radix must divide the elements per thread");
   constexpr int NB = E / R;
   constexpr bool LAST = sizeof...(REST) == 0;
@@ -41,10 +47,17 @@ __device__ __forceinline__ void rfft_stages(float2 (&x)[E], const int i, const f
   for (int u = 0; u < NB; ++u) {
     const int ib = i + (L / E) * u;
     const int k = ib & (P - 1);
-    float2 z[R];
+    V z[R];
 #pragma unroll
     for (int m = 0; m < R; ++m) z[m] = x[u + m * NB];
-    if constexpr (P > 1) {
+    if constexpr (P > 1 && sizeof(T) == 8) {
+      const int b = k * (L / (P * R));
+#pragma unroll
+      for (int m = 1; m < R; ++m) {
+        const V w = __ldg(tw + m * b);
+        z[m] = SIGN > 0 ? cmulc(z[m], w) : cmul(z[m], w);
+      }
+    } else if constexpr (P > 1) {
       // one or four L1 loads per butterfly instead of R - 1, the rest on the FP32 pipe
       const int b = k * (L / (P * R));
 #if CMM_TW_MODE == 1
@@ -71,7 +84,7 @@ __device__ __forceinline__ void rfft_stages(float2 (&x)[E], const int i, const f
       for (int m = 1; m < R; ++m) z[m] = cmul(z[m], wp[m]);
 #endif
     }
-    dft_reg<float, clog2(R), SIGN>(z);
+    dft_reg<T, clog2(R), SIGN>(z);
     if constexpr (LAST) {
 #pragma unroll
       for (int q = 0; q < R; ++q) x[u + q * NB] = z[q];
@@ -87,13 +100,13 @@ __device__ __forceinline__ void rfft_stages(float2 (&x)[E], const int i, const f
     const int b = ad.base(i);
 #pragma unroll
     for (int e = 0; e < E; ++e) x[e] = ad.ld_at(b, e * (L / E));
-    rfft_stages<SIGN, E, L, P * R, Addr, REST...>(x, i, tw, ad);
+    rfft_stages<SIGN, E, L, P * R, V, Addr, REST...>(x, i, tw, ad);
   }
 }
 
-template <int SIGN, int E, int... RS, typename Addr>
-__device__ __forceinline__ void rfft(float2 (&x)[E], const int i, const float2* __restrict__ tw, const Addr& ad) {
-  rfft_stages<SIGN, E, RadProd<RS...>::value, 1, Addr, RS...>(x, i, tw, ad);
+template <int SIGN, int E, int... RS, typename V, typename Addr>
+__device__ __forceinline__ void rfft(V (&x)[E], const int i, const V* __restrict__ tw, const Addr& ad) {
+  rfft_stages<SIGN, E, RadProd<RS...>::value, 1, V, Addr, RS...>(x, i, tw, ad);
 }
 
 // One contiguous row (pass F), padded by one element every 2^PS positions.
@@ -148,12 +161,19 @@ template <typename T, int SIGN>
 __device__ __forceinline__ Cx2<T> cx_rot32(const Cx2<T>& v, int m) {
   m &= 31;
   if (m == 0) return v;
-  const V2<T> zero{(T)0, (T)0};
-  const Cx2<T> pos{psub(zero, v.im), v.re}, neg{v.im, psub(zero, v.re)};   // i v, -i v
+  const Cx2<T> pos{V2<T>{-v.im.x, -v.im.y}, v.re}, neg{v.im, V2<T>{-v.re.x, -v.re.y}};   // i v, -i v
   if (m == 8) return SIGN < 0 ? neg : pos;
   if (m == 24) return SIGN < 0 ? pos : neg;
-  if (m == 16) return Cx2<T>{psub(zero, v.re), psub(zero, v.im)};
+  if (m == 16) return Cx2<T>{V2<T>{-v.re.x, -v.re.y}, V2<T>{-v.im.x, -v.im.y}};
   return cx_mul<T>(v, (T)cos32(m), (T)(SIGN * sin32(m)));
+}
+
+// a + SIGN i b and a - SIGN i b: parts swapped by name, no instruction of their own
+template <typename T, int SIGN>
+__device__ __forceinline__ void cx_addsub_i(const Cx2<T>& a, const Cx2<T>& b, Cx2<T>& plus, Cx2<T>& minus) {
+  const Cx2<T> p{psub(a.re, b.im), padd(a.im, b.re)}, m{padd(a.re, b.im), psub(a.im, b.re)};
+  plus = SIGN > 0 ? p : m;
+  minus = SIGN > 0 ? m : p;
 }
 
 template <typename T, int SIGN>
@@ -161,21 +181,29 @@ __device__ __forceinline__ void cx_dft4(Cx2<T>& x0, Cx2<T>& x1, Cx2<T>& x2, Cx2<
   const Cx2<T> a0 = cx_add(x0, x2), a1 = cx_sub(x0, x2), a2 = cx_add(x1, x3), d = cx_sub(x1, x3);
   x0 = cx_add(a0, a2);
   x2 = cx_sub(a0, a2);
-  // a1 +- SIGN i d: parts of d swapped by name, no instruction of their own
-  if (SIGN < 0) {
-    x1 = Cx2<T>{padd(a1.re, d.im), psub(a1.im, d.re)};
-    x3 = Cx2<T>{psub(a1.re, d.im), padd(a1.im, d.re)};
-  } else {
-    x1 = Cx2<T>{psub(a1.re, d.im), padd(a1.im, d.re)};
-    x3 = Cx2<T>{padd(a1.re, d.im), psub(a1.im, d.re)};
-  }
+  cx_addsub_i<T, SIGN>(a1, d, x1, x3);
 }
 
-// x_q <- sum_j x_j w_R^{j q}, R = 2^LR <= 16 (4 x 4 for 16, else radix-2 stages)
+// x_q <- sum_j x_j w_R^{j q}, R = 2^LR <= 16 (4 x 4 for 16, 4 x 2 for 8, else radix-2 stages)
 template <typename T, int LR, int SIGN>
 __device__ __forceinline__ void cx_dft(Cx2<T>* x) {
   if constexpr (LR == 2) {
     cx_dft4<T, SIGN>(x[0], x[1], x[2], x[3]);
+  } else if constexpr (LR == 3) {
+    Cx2<T> e[4] = {x[0], x[2], x[4], x[6]}, o[4] = {x[1], x[3], x[5], x[7]};
+    cx_dft4<T, SIGN>(e[0], e[1], e[2], e[3]);
+    cx_dft4<T, SIGN>(o[0], o[1], o[2], o[3]);
+    o[1] = cx_rot32<T, SIGN>(o[1], 4);
+    o[3] = cx_rot32<T, SIGN>(o[3], 12);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (k == 2) {
+        cx_addsub_i<T, SIGN>(e[2], o[2], x[2], x[6]);
+      } else {
+        x[k] = cx_add(e[k], o[k]);
+        x[k + 4] = cx_sub(e[k], o[k]);
+      }
+    }
   } else if constexpr (LR == 4) {
 #pragma unroll
     for (int n1 = 0; n1 < 4; ++n1) cx_dft4<T, SIGN>(x[n1], x[n1 + 4], x[n1 + 8], x[n1 + 12]);
@@ -233,7 +261,14 @@ __device__ __forceinline__ void rfft2_stages(Cx2<T> (&x)[E], const int i, const 
     Cx2<T> z[R];
 #pragma unroll
     for (int m = 0; m < R; ++m) z[m] = x[u + m * NB];
-    if constexpr (P > 1) {
+    if constexpr (P > 1 && sizeof(T) == 8) {
+      const int b = k * (L / (P * R));
+#pragma unroll
+      for (int m = 1; m < R; ++m) {
+        const V2<T> w = __ldg(tw + m * b);
+        z[m] = cx_mul<T>(z[m], w.x, SIGN > 0 ? -w.y : w.y);
+      }
+    } else if constexpr (P > 1) {
       const int b = k * (L / (P * R));
       V2<T> w1 = __ldg(tw + b);
       if (SIGN > 0) w1.y = -w1.y;

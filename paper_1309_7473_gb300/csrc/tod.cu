@@ -434,7 +434,7 @@ static int prepare_nc(int prec) {
 // (done once, before any stream capture).
 int op_prepare_kernels(cmm_op* op) {
   if (fast_path_ok(op)) CMM_TRY(prepare_fast(op));
-  if (op->prec != CMM_PREC_F64) CMM_TRY(prepare_pair(op));
+  CMM_TRY(prepare_pair(op));
   return op->pt->ncomp == 1 ? prepare_nc<1>(op->prec) : prepare_nc<3>(op->prec);
 }
 

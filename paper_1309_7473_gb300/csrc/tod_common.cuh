@@ -78,6 +78,8 @@ struct TodArgs {
   const int4* bore;
   const int2* det_off;
   const float2* rot2;   // [n_t] (cos 2phi, sin 2phi) in FP32
+  const double2* rot64; // [n_t] (cos 2phi, sin 2phi) in FP64 (FP64 two-detector path)
+  const double* lg2;    // [n_t / 2 + 1] log2 of the frequency index (of 1 at 0), then 2^(j / 64), j < 64 (the same)
   const void* pol;      // V2<T> [n_det]
   const void* coef;     // V4<T> [n_det]
   const void* wtab;     // T [n_det][N + 1] tabulated w_d(f_k), or nullptr (the parametric law)
@@ -163,6 +165,8 @@ static inline TodArgs make_args(const cmm_op* op, int d0) {
   a.bore = pt->bore;
   a.det_off = pt->det_off;
   a.rot2 = pt->rot2;
+  a.rot64 = op->rot64;
+  a.lg2 = op->lg2;
   const bool f64 = op->prec == CMM_PREC_F64;
   a.pol = f64 ? (const void*)pt->det_pol64 : (const void*)pt->det_pol32;
   a.coef = f64 ? (const void*)op->nz->coef64 : (const void*)op->nz->coef32;

@@ -94,41 +94,42 @@ __device__ __forceinline__ int pixel_fast(const int4 b, const int2 o, int ny, in
 }
 
 // w_N^e, 0 <= e < N, from the two tables w_N^(e mod C) and w_R^(e div C)
-__device__ __forceinline__ float2 tw_N(const TodArgs& a, const float2* __restrict__ tw, int e) {
-  const float2 lo = __ldg(tw + a.twl.Nlo_off + (e & (a.C - 1)));
-  const float2 hi = __ldg(tw + a.twl.R_off + (e >> a.logC));
+template <typename V>
+__device__ __forceinline__ V tw_N(const TodArgs& a, const V* __restrict__ tw, int e) {
+  const V lo = __ldg(tw + a.twl.Nlo_off + (e & (a.C - 1)));
+  const V hi = __ldg(tw + a.twl.R_off + (e >> a.logC));
   return cmul(lo, hi);
 }
 
 // J interleaved columns: position pos of column cl at J pos + cl, so every access
 // of the column FFT puts consecutive lanes on consecutive elements.
-template <int J>
+template <int J, typename V = float2>
 struct ColJ {
-  float2* buf;
+  V* buf;
   int cl;
-  __device__ __forceinline__ void st(int pos, float2 v) const { buf[pos * J + cl] = v; }
-  __device__ __forceinline__ float2 ld(int pos) const { return buf[pos * J + cl]; }
+  __device__ __forceinline__ void st(int pos, V v) const { buf[pos * J + cl] = v; }
+  __device__ __forceinline__ V ld(int pos) const { return buf[pos * J + cl]; }
   __device__ __forceinline__ int base(int pos) const { return pos * J + cl; }
-  __device__ __forceinline__ void st_at(int b, int o, float2 v) const { buf[b + o * J] = v; }
-  __device__ __forceinline__ float2 ld_at(int b, int o) const { return buf[b + o * J]; }
+  __device__ __forceinline__ void st_at(int b, int o, V v) const { buf[b + o * J] = v; }
+  __device__ __forceinline__ V ld_at(int b, int o) const { return buf[b + o * J]; }
 };
 
 template <int R> struct ColPlan;
 template <> struct ColPlan<64> {
-  template <int SIGN, typename Addr>
-  static __device__ __forceinline__ void run(float2 (&x)[kE], int i, const float2* tw, const Addr& ad) {
+  template <int SIGN, typename V, typename Addr>
+  static __device__ __forceinline__ void run(V (&x)[kE], int i, const V* tw, const Addr& ad) {
     rfft<SIGN, kE, 16, 4>(x, i, tw, ad);
   }
 };
 template <> struct ColPlan<128> {
-  template <int SIGN, typename Addr>
-  static __device__ __forceinline__ void run(float2 (&x)[kE], int i, const float2* tw, const Addr& ad) {
+  template <int SIGN, typename V, typename Addr>
+  static __device__ __forceinline__ void run(V (&x)[kE], int i, const V* tw, const Addr& ad) {
     rfft<SIGN, kE, 16, 8>(x, i, tw, ad);
   }
 };
 template <> struct ColPlan<256> {
-  template <int SIGN, typename Addr>
-  static __device__ __forceinline__ void run(float2 (&x)[kE], int i, const float2* tw, const Addr& ad) {
+  template <int SIGN, typename V, typename Addr>
+  static __device__ __forceinline__ void run(V (&x)[kE], int i, const V* tw, const Addr& ad) {
     rfft<SIGN, kE, 16, 16>(x, i, tw, ad);
   }
 };
