@@ -228,8 +228,8 @@ bool fast_path_sizes(int logN, int prec, int* logR, int* logC);
 bool pair_path_fits(const cmm_op* op);
 bool pair_path_ok(const cmm_op* op);
 bool pair_path_sizes(int log_nt, int* logR, int* logC);
-int launch_apply_chunk_pair(cmm_op* op, int d0, int nd, int pass);
-int launch_apply_chunk_pair64(cmm_op* op, int d0, int nd, int pass);
+int launch_apply_chunk_pair(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, int pass);
+int launch_apply_chunk_pair64(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, int pass);
 int prepare_pair(cmm_op* op);
 int prepare_pair64(cmm_op* op);
 

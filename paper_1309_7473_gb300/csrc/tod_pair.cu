@@ -26,13 +26,15 @@ int launch_flush(const TodArgs& a, int nc, cudaStream_t st);
 int launch_flush_maps(const TodArgs& a, int nc, int maps, cudaStream_t st);
 
 template <typename S>
-static int apply_pair_s(cmm_op* op, int d0, int nd, int pass) {
+static int apply_pair_s(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, int pass) {
   TodArgs a = pair_args(op, d0);
+  a.tod = tod;
   cudaStream_t st = op->ctx->stream;
   const int nc = op->pt->ncomp;
   if (pass < 0 || pass == 0) {
     TraceRange tr("A: P m + column FFTs (two detectors per sequence)");
-    if (nc == 1) CMM_TRY((dispatch_pair_T<float, 1, S>(a, nd, 0, st, false)));
+    if (tod) CMM_TRY((dispatch_pair_D<float, S>(a, nd, tod_is_f64 != 0, st, false)));
+    else if (nc == 1) CMM_TRY((dispatch_pair_T<float, 1, S>(a, nd, 0, st, false)));
     else CMM_TRY((dispatch_pair_T<float, 3, S>(a, nd, 0, st, false)));
   }
   if (pass < 0 || pass == 1) {
@@ -59,10 +61,11 @@ static int apply_pair_s(cmm_op* op, int d0, int nd, int pass) {
   return CMM_OK;
 }
 
-int launch_apply_chunk_pair(cmm_op* op, int d0, int nd, int pass) {
-  if (op->prec == CMM_PREC_F64) return launch_apply_chunk_pair64(op, d0, nd, pass);
-  if (op->prec == CMM_PREC_BF16) return apply_pair_s<__nv_bfloat162>(op, d0, nd, pass);
-  return apply_pair_s<float2>(op, d0, nd, pass);
+// tod: stored data [n_det][n_t] in place of P m, or nullptr.
+int launch_apply_chunk_pair(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, int pass) {
+  if (op->prec == CMM_PREC_F64) return launch_apply_chunk_pair64(op, d0, nd, tod, tod_is_f64, pass);
+  if (op->prec == CMM_PREC_BF16) return apply_pair_s<__nv_bfloat162>(op, d0, nd, tod, tod_is_f64, pass);
+  return apply_pair_s<float2>(op, d0, nd, tod, tod_is_f64, pass);
 }
 
 // The split, which n_samp fixes, its tables and the kernels' shared-memory attributes.

@@ -61,3 +61,21 @@ def test_table(cmm):
     scan = gen.small_scan(cfg=393, ny=24, nx=20, n_t=1 << 13, ncols=3, nrows=1, throw_px=30.0)
     w = 1.0 + 0.5 * np.sin(np.arange(scan.n_t // 2 + 1) / 7.0)[None] * np.array([[0.2], [0.9], [0.5]])
     assert max(both(cmm, scan, gen.noise_params(3), w)) < 1e-11
+
+
+@pytest.mark.parametrize("prec,tol", [(0, 1e-11), (1, 1e-5)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("log_nt,n_det,ncomp", [(13, 1, 1), (15, 5, 3), (16, 8, 3), (18, 3, 3)])
+def test_rhs_of_stored_data(cmm, prec, tol, dtype, log_nt, n_det, ncomp):
+    """The right-hand side on the two-detector path against the one-detector kernels
+    (FP32: the operator's bound; the data are white, so no large offsets are filtered)."""
+    full = gen.small_scan(cfg=394, ny=30, nx=32, n_t=1 << log_nt, ncols=4, nrows=2, throw_px=40.0, ncomp=ncomp)
+    scan = full.subset(np.arange(n_det))
+    op = cmm.Operator(cmm.Context(0), scan, gen.noise_params(n_det, scatter=0.2, cfg=394), precision=prec)
+    g = torch.Generator(device="cuda:0").manual_seed(394)
+    tod = torch.randn((n_det, scan.n_t), dtype=dtype, device="cuda:0", generator=g)
+    pair = op.rhs(tod).clone()
+    op.set_pair_packing(False)
+    ref = op.rhs(tod)
+    assert float((pair - ref).norm()) <= tol * float(ref.norm())
+    assert float((pair - ref).abs().max()) <= tol * float(ref.abs().max())
