@@ -21,6 +21,7 @@
 #include "common.cuh"
 #include "fft.cuh"
 #include "tod_common.cuh"
+#include "tod_fast.cuh"
 
 namespace cmm {
 
@@ -212,15 +213,54 @@ __global__ void k_acc_to_map(const double* __restrict__ acc, const uint8_t* __re
   }
 }
 
-// tod[d][t] = (P m)_{d,t}: pointing + gather only (used to synthesise noise-free data)
-template <typename T, int NC, typename OUT>
-__global__ void k_project(const TodArgs a, OUT* __restrict__ tod) {
-  const int d = blockIdx.y;
-  const int2 off = a.det_off[d];
-  const V2<T> pol = reinterpret_cast<const V2<T>*>(a.pol)[d];
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < a.n_t;
-       t += (long long)gridDim.x * blockDim.x)
-    tod[(long long)d * a.n_t + t] = (OUT)project_sample<T, NC>(a, off, pol, t);
+// tod[d][t] = (P m)_{d,t}: pointing + gather only (used to synthesise noise-free data).
+// Bound by the stores once the sample's own work is shared: a thread keeps kProjSamples
+// samples (boresight and rotation in registers, the rotation from the FP32 table or, in
+// FP64, by its two divisions once) and takes them through kProjDets detectors; lanes stay
+// on consecutive samples, which fall on a third as many pixels.  512 x 2^19 samples in
+// FP32: 831 -> 361 us with the map copy (one sample and detector a thread before, with
+// two divisions each); 1.1 GB of stores take 159 us.
+constexpr int kProjSamples = 4, kProjDets = 8, kProjThreads = 256;
+
+template <typename T, int NC, typename OUT, bool PERIODIC>
+__global__ void __launch_bounds__(kProjThreads) k_project(const TodArgs a, OUT* __restrict__ tod, int n_det) {
+  const int t0 = blockIdx.x * (kProjThreads * kProjSamples) + threadIdx.x;
+  const int npix = (int)a.npix, n_t = (int)a.n_t;
+  int4 b[kProjSamples];
+  V2<T> r[kProjSamples];
+#pragma unroll
+  for (int k = 0; k < kProjSamples; ++k) {
+    const int t = min(t0 + k * kProjThreads, n_t - 1);
+    b[k] = __ldg(a.bore + t);
+    if constexpr (NC == 3 && sizeof(T) == 4) {
+      const float2 v = __ldg(a.rot2 + t);
+      r[k] = V2<T>{v.x, v.y};
+    } else if constexpr (NC == 3) {
+      sample_response<T>(b[k], V2<T>{(T)1, (T)0}, r[k].x, r[k].y);
+    }
+  }
+  const int d1 = min(n_det, (int)(blockIdx.y + 1) * kProjDets);
+#pragma unroll 2
+  for (int d = blockIdx.y * kProjDets; d < d1; ++d) {
+    const int2 off = a.det_off[d];
+    const V2<T> pol = reinterpret_cast<const V2<T>*>(a.pol)[d];
+    OUT* row = tod + (size_t)d * n_t;
+#pragma unroll
+    for (int k = 0; k < kProjSamples; ++k) {
+      const int t = t0 + k * kProjThreads;
+      const int p = pixel_fast<PERIODIC>(b[k], off, a.ny, a.nx, npix);   // npix, outside: zero
+      T v;
+      if constexpr (NC == 1) {
+        v = reinterpret_cast<const T*>(a.gather)[p];
+      } else {
+        const V4<T> g = reinterpret_cast<const V4<T>*>(a.gather)[p];
+        const T c = pol.x * r[k].x - pol.y * r[k].y;
+        const T s = pol.y * r[k].x + pol.x * r[k].y;
+        v = g.x + c * g.y + s * g.z;
+      }
+      if (t < n_t) __stcs(row + t, (OUT)v);
+    }
+  }
 }
 
 // Per-pixel blocks sum_t u_d P_t P_t^T (Eq. 3-5): [npix][6] = (TT, TQ, TU, QQ, QU, UU)
@@ -474,14 +514,17 @@ int launch_generic_fwd_from_tod(cmm_op* op, int d0, int nd, const void* tod, int
 
 template <typename T, int NC>
 static int project_t(cmm_op* op, void* tod, int tod_is_f64) {
-  TodArgs a = make_args(op, 0);
-  const long long n_t = op->pt->n_t;
-  const int bx = (int)std::min<long long>((n_t + 255) / 256, 1024);
-  dim3 g(bx, op->pt->n_det);
-  if (tod_is_f64)
-    k_project<T, NC, double><<<g, 256, 0, op->ctx->stream>>>(a, (double*)tod);
-  else
-    k_project<T, NC, float><<<g, 256, 0, op->ctx->stream>>>(a, (float*)tod);
+  const TodArgs a = make_args(op, 0);
+  const int n_det = op->pt->n_det, per = kProjThreads * kProjSamples;
+  const dim3 g((unsigned)((op->pt->n_t + per - 1) / per), (n_det + kProjDets - 1) / kProjDets);
+  cudaStream_t st = op->ctx->stream;
+  if (tod_is_f64) {
+    if (a.periodic) k_project<T, NC, double, true><<<g, kProjThreads, 0, st>>>(a, (double*)tod, n_det);
+    else k_project<T, NC, double, false><<<g, kProjThreads, 0, st>>>(a, (double*)tod, n_det);
+  } else {
+    if (a.periodic) k_project<T, NC, float, true><<<g, kProjThreads, 0, st>>>(a, (float*)tod, n_det);
+    else k_project<T, NC, float, false><<<g, kProjThreads, 0, st>>>(a, (float*)tod, n_det);
+  }
   CMM_LAUNCH_CHECK();
   return CMM_OK;
 }
