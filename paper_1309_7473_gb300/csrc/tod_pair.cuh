@@ -58,9 +58,6 @@
 namespace cmm {
 
 // Tuning knobs of this path (compile-time; the defaults are the measured best).
-#ifndef CMM_PAIR_XOR
-#define CMM_PAIR_XOR 1     // pixel staging: 0 = rows padded to J + 8 ints, 1 = XOR-swizzled 16-byte chunks (no pad)
-#endif
 
 // A binning run in the frame of the scan rotation: for samples of one detector on
 // one pixel, sums of u, u cos 2phi_t and u sin 2phi_t; the detector angle psi_d
@@ -97,12 +94,18 @@ __device__ __forceinline__ void pair_run_close(double* acc, const PairRun<double
   }
 }
 
-// Launch shapes: the FP32 column shapes of tod_fast.cuh, and one block per SM in FP64
-// (64 KB tiles; one warp instruction in 16 cycles keeps its pipe full with few warps).
-template <typename T, int R> struct PairShape : ColShape<R> {};
+// Launch shapes: 16 columns a block, so that half a warp reads 16 consecutive samples (32
+// columns at R <= 128 left too few blocks to balance: A at 128 x 2^17 149 against 143 us),
+// for 32 resident warps per SM forward and 24 in the binning.  FP64: 8 columns, small
+// blocks of a pipe that few warps fill (A at 32 x 2^16: 395 us, 405 with 32 columns).
+template <typename T, int R> struct PairShape {
+  static constexpr int J = 16;
+  static constexpr int THREADS = J * R / kE;
+  static constexpr int MINB = 1024 / THREADS, MINB_INV = 768 / THREADS;
+};
 template <int R> struct PairShape<double, R> {
-  static constexpr int J = ColShape<R>::J;
-  static constexpr int THREADS = ColShape<R>::THREADS;
+  static constexpr int J = 8;
+  static constexpr int THREADS = J * R / kE;
   static constexpr int MINB = 1, MINB_INV = 1;
 };
 
@@ -322,7 +325,8 @@ __global__ void __launch_bounds__(PairShape<T, R>::THREADS, PairShape<T, R>::MIN
 // FP64: 8 points of both rows a thread and one block per SM.
 template <typename T, int C, int E> struct PairFilterShape {
   static constexpr int TPR = C / E;   // threads per row pair
-  static constexpr int THREADS = TPR > 128 ? TPR : 128;
+  static constexpr int LEAST = sizeof(T) == 8 ? 32 : 128;
+  static constexpr int THREADS = TPR > LEAST ? TPR : LEAST;
   static constexpr int PAIRS = THREADS / TPR;   // row pairs per CTA
   static constexpr int MINB = sizeof(T) == 8 ? 1 : 512 / THREADS;
 };
@@ -414,11 +418,10 @@ __global__ void __launch_bounds__(PairShape<T, R>::THREADS, PairShape<T, R>::MIN
   constexpr int SPL = 8;              // consecutive samples per lane
   constexpr int LPR = J / SPL;        // lanes per row
   constexpr int RPP = NT / LPR;       // rows per binning pass
-  // Pixel staging: row stride PS ints; a lane's 8 pixels are two 16-byte chunks
-  // interleaved with its row neighbour's (chunk h of lane bq at word 8h + 4bq of a
-  // 16-sample group), so that the eight lanes of a quarter-warp load hit eight
-  // distinct 4-bank groups (PS = 24 words = 8 mod 32 shifts consecutive rows).
-  constexpr int PS = CMM_PAIR_XOR ? J + (J == 32 ? 8 : 0) : J + 8;
+  // Pixel staging: rows of PS ints; a lane's 8 pixels are two 16-byte chunks interleaved
+  // with its row neighbour's and permuted by an XOR with the row, so that the staging
+  // stores and the eight lanes of a quarter-warp load spread over the 4-bank groups.
+  constexpr int PS = 16;
   static_assert(LPR >= 1 && RPP <= R && R % RPP == 0 && (RPP * J) % NT == 0, "binning layout");
   if (a.done && *a.done) return;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -492,10 +495,8 @@ __global__ void __launch_bounds__(PairShape<T, R>::THREADS, PairShape<T, R>::MIN
         const int sidx = threadIdx.x + k * NT;
         const int rr = sidx / J, col = sidx % J;
         const int4 b = __ldg(a.bore + c0 + col + (kr0 + rr) * a.C);
-        // column col = 16 g + 8 bq + 4 h + w of the row goes to word 16 g + 8 h + 4 bq + w
-        // (padded rows), or to chunk (2 h + bq) ^ (row & 3) of its 16-word group
-        const int sw = CMM_PAIR_XOR ? (col & ~15) | (((((col >> 1) & 2) | ((col >> 3) & 1)) ^ (rr & 3)) << 2) | (col & 3)
-                                    : (col & ~15) | ((col & 4) << 1) | ((col & 8) >> 1) | (col & 3);
+        // column col = 8 bq + 4 h + w of the row goes to chunk (2 h + bq) ^ (row & 3)
+        const int sw = (((((col >> 1) & 2) | ((col >> 3) & 1)) ^ (rr & 3)) << 2) | (col & 3);
         pst[rr * PS + sw] = pixel_fast<PERIODIC>(b, off1, a.ny, a.nx, npix);
         pst[(RPP + rr) * PS + sw] = pixel_fast<PERIODIC>(b, off2, a.ny, a.nx, npix);
       }
@@ -529,17 +530,9 @@ __global__ void __launch_bounds__(PairShape<T, R>::THREADS, PairShape<T, R>::MIN
         P0 = __ldcs(reinterpret_cast<const int4*>(pixd));
         P1 = __ldcs(reinterpret_cast<const int4*>(pixd + 4));
       } else {
-        const int* prow = pst + (dd * RPP + br) * PS + ((bq >> 1) << 4);
-        if (CMM_PAIR_XOR) {
-          // chunks (2 h + bq % 2) ^ (row & 3) of the 16-word group
-          P0 = *reinterpret_cast<const int4*>(prow + (((bq & 1) ^ (br & 3)) << 2));
-          P1 = *reinterpret_cast<const int4*>(prow + (((2 | (bq & 1)) ^ (br & 3)) << 2));
-        } else {
-          // chunks h = 0, 1 of the lane's 8 pixels at words 16 (bq / 2) + 4 (bq % 2) + 8 h
-          const int4* ps = reinterpret_cast<const int4*>(prow + ((bq & 1) << 2));
-          P0 = ps[0];
-          P1 = ps[2];
-        }
+        const int* prow = pst + (dd * RPP + br) * PS;
+        P0 = *reinterpret_cast<const int4*>(prow + ((bq ^ (br & 3)) << 2));
+        P1 = *reinterpret_cast<const int4*>(prow + (((2 | bq) ^ (br & 3)) << 2));
       }
       p[0] = P0.x; p[1] = P0.y; p[2] = P0.z; p[3] = P0.w;
       p[4] = P1.x; p[5] = P1.y; p[6] = P1.z; p[7] = P1.w;
@@ -572,12 +565,11 @@ template <typename T, int NC, typename S, int R, bool PERIODIC, bool CACHED>
 inline int run_pair_T_c(const TodArgs& a, int nd, int pass, cudaStream_t st, bool attr_only) {
   constexpr int J = PairShape<T, R>::J;
   constexpr int NT = PairShape<T, R>::THREADS;
-  // forward: FFT tile R x J complex.  inverse: binning tile R x (J + 2) complex, the
-  // pixel staging of one pass (2 detectors x RPP rows x (J + 8) ints) and, when the
-  // rotation is staged, RPP rows x (J + 2) complex
+  // forward: FFT tile R x J complex.  inverse: binning tile R x (J + 2) complex and the
+  // pixel staging of one pass (2 detectors x RPP rows x PS ints)
   constexpr int RPP = NT / (J / 8);   // rows per binning pass
   const int smem_f = (int)(sizeof(V2<T>) * R * J);
-  constexpr int PS = CMM_PAIR_XOR ? J + (J == 32 ? 8 : 0) : J + 8;
+  constexpr int PS = 16;
   // (the pixel-cache instances stage no pixels: less shared memory leaves more L1)
   const int smem_i = (int)(sizeof(V2<T>) * R * (J + 2) + (CACHED ? 0 : sizeof(int) * 2 * RPP * PS));
   if (attr_only) {
@@ -660,9 +652,12 @@ template <typename T, typename S>
 inline int dispatch_pair_F(const TodArgs& a, int nd, cudaStream_t st, bool attr_only) {
   if constexpr (sizeof(T) == 4) {
     switch (a.logC) {
-      case 7: return run_pair_F<T, S, 16, 16, 8>(a, nd, st, attr_only);
-      case 8: return run_pair_F<T, S, 16, 16, 16>(a, nd, st, attr_only);
-      case 9: return run_pair_F<T, S, 16, 16, 16, 2>(a, nd, st, attr_only);
+      // short rows: 8 points a thread, twice the threads (row transforms of 32 x 2^16 take
+      // 10.3 against 12.4 us); from 1024 points on the third exchange costs more (75
+      // against 74 us at 1024, 2.82 against 2.45 ms at 4096)
+      case 7: return run_pair_F<T, S, 8, 8, 8, 2>(a, nd, st, attr_only);
+      case 8: return run_pair_F<T, S, 8, 8, 8, 4>(a, nd, st, attr_only);
+      case 9: return run_pair_F<T, S, 8, 8, 8, 8>(a, nd, st, attr_only);
       case 10: return run_pair_F<T, S, 16, 16, 16, 4>(a, nd, st, attr_only);
       case 11: return run_pair_F<T, S, 16, 16, 16, 8>(a, nd, st, attr_only);
       case 12: return run_pair_F<T, S, 16, 16, 16, 16>(a, nd, st, attr_only);

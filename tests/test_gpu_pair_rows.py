@@ -22,7 +22,7 @@ def cmm():
     return c
 
 
-@pytest.mark.parametrize("log_nt,R", [(13, 64), (16, 128), (18, 256)])
+@pytest.mark.parametrize("log_nt,R", [(13, 64), (14, 64), (16, 128), (17, 128), (18, 256)])
 @pytest.mark.parametrize("rows", ["zero", "half", "one", "last"])
 @pytest.mark.parametrize("n_det", [1, 3])
 def test_rows_by_themselves(cmm, log_nt, R, rows, n_det):
