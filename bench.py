@@ -456,7 +456,9 @@ def run_ours(args, rank, world):
         "setup_seconds": round(setup_s, 2),
         "clocks": clocks,
     }
-    out["gpu_launches"] = (launches_per_iteration(scan.n_det, chunk_dets, CIRC_FUSED_LAUNCHES) * args.steps
+    # the FP32 two-detector path: the application's last flush writes the map
+    map_out = 0 if args.prec != "f64" and args.corr_modes == 0 else 1
+    out["gpu_launches"] = (launches_per_iteration(scan.n_det, chunk_dets, CIRC_FUSED_LAUNCHES, map_out) * args.steps
                            + SETUP_LAUNCHES + CIRC_FUSED_LAUNCHES)
     return out
 
@@ -653,14 +655,14 @@ def cufft_filter_ms(scan, noise, dev, stream):
                     "excludes P and P^T", "ms": ms}
 
 
-def launches_per_iteration(n_det, chunk, circ=None):
+def launches_per_iteration(n_det, chunk, circ=None, map_out=1):
     """Kernels of one circulant-PCG iteration: the A-application (map copy in, per
     chunk one forward and one filter launch and, per 2048 detectors (eight FP32
-    partial maps of 256 detectors), one inverse + binning launch and one flush; map
-    copy out), the CG update kernels and the circulant preconditioner: `circ`
+    partial maps of 256 detectors), one inverse + binning launch and one flush; a map
+    copy out where the flush does not write the map), the CG update kernels and the circulant preconditioner: `circ`
     kernels, by default those of the maps that the line FFTs serve (Sigma^-1,
     2-D FFTs, per-mode solve)."""
-    a = 2
+    a = 1 + map_out
     maps = min(8, max(1, math.ceil(chunk / 256)))
     for d0 in range(0, n_det, chunk):
         nd = min(chunk, n_det - d0)

@@ -639,12 +639,7 @@ extern "C" {
 
 static int apply_A_dev(cmm_op* op, const double* m_in, double* m_out) {
   TraceRange tr("cmm: A = P^T N^-1 P");
-  CMM_TRY(launch_map_to_gather(op, m_in));
-  for (int d0 = 0; d0 < op->pt->n_det; d0 += op->chunk) {
-    const int nd = std::min(op->chunk, op->pt->n_det - d0);
-    CMM_TRY(launch_apply_chunk(op, d0, nd, nullptr, 0));
-  }
-  return launch_acc_to_map(op, m_out);
+  return launch_apply(op, m_in, nullptr, 0, m_out);
 }
 
 int cmm_apply_A(cmm_op* op, const double* m_in, double* m_out) {
@@ -669,16 +664,16 @@ int cmm_profile_apply(cmm_op* op, const double* m_in, double* m_out, int32_t rep
     int k = 0;
     CMM_CUDA(cudaEventRecord(ev[k++], st));
     for (int r = 0; r < reps; ++r) {
-      CMM_TRY(launch_map_to_gather(op, m_in));
+      CMM_TRY(launch_map_to_gather(op, m_in, apply_uses_acc(op)));
       CMM_CUDA(cudaEventRecord(ev[k++], st));
       for (int d0 = 0; d0 < op->pt->n_det; d0 += op->chunk) {
         const int nd = std::min(op->chunk, op->pt->n_det - d0);
         for (int pass = 0; pass < 3; ++pass) {
-          CMM_TRY(launch_apply_chunk(op, d0, nd, nullptr, 0, pass));
+          CMM_TRY(launch_apply_chunk(op, d0, nd, nullptr, 0, m_out, pass));
           CMM_CUDA(cudaEventRecord(ev[k++], st));
         }
       }
-      CMM_TRY(launch_acc_to_map(op, m_out));
+      if (!apply_direct(op)) CMM_TRY(launch_acc_to_map(op, m_out));
       CMM_CUDA(cudaEventRecord(ev[k++], st));
     }
     CMM_CUDA(cudaEventRecord(ev[k++], st));
@@ -736,12 +731,7 @@ int cmm_rhs(cmm_op* op, const void* tod, int32_t tod_is_f64, double* b) {
   if (!op || !tod || !b) return fail(CMM_ERR_ARG, "null argument");
   CMM_CUDA(cudaSetDevice(op->ctx->device));
   CMM_TRY(op_sync_corr(op));
-  CMM_CUDA(cudaMemsetAsync(op->acc, 0, sizeof(double) * op->acc_stride * op->pt->npix, op->ctx->stream));
-  for (int d0 = 0; d0 < op->pt->n_det; d0 += op->chunk) {
-    const int nd = std::min(op->chunk, op->pt->n_det - d0);
-    CMM_TRY(launch_apply_chunk(op, d0, nd, tod, tod_is_f64));
-  }
-  return launch_acc_to_map(op, b);
+  return launch_apply(op, nullptr, tod, tod_is_f64, b);
 }
 
 int cmm_dot(cmm_op* op, const double* x, const double* y, int64_t n, double* result_host) {

@@ -351,9 +351,9 @@ __global__ void __launch_bounds__(CircKernel<T>::kRowThreads, CircKernel<T>::kRo
           const V2<T>* b = reinterpret_cast<const V2<T>*>(br) + 3 * pos;
           const V2<T> b0 = b[0], b1 = b[1], b2 = b[2];
           const T x0 = v.re.x * sc, x1 = v.im.x * sc, x2 = v.re.y * sc;
-          const double y0 = (double)(b0.x * x0 + b0.y * x1 + b1.x * x2);
-          const double y1 = (double)(b0.y * x0 + b1.y * x1 + b2.x * x2);
-          const double y2 = (double)(b1.x * x0 + b2.x * x1 + b2.y * x2);
+          const double y0 = widen(b0.x * x0 + b0.y * x1 + b1.x * x2);
+          const double y1 = widen(b0.y * x0 + b1.y * x1 + b2.x * x2);
+          const double y2 = widen(b1.x * x0 + b2.x * x1 + b2.y * x2);
           zr[pos] = y0;
           zr[npix + pos] = y1;
           zr[2 * npix + pos] = y2;

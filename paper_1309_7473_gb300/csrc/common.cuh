@@ -84,6 +84,16 @@ __device__ __forceinline__ double2 padd(double2 a, double2 b) { return double2{a
 __device__ __forceinline__ double2 psub(double2 a, double2 b) { return double2{a.x - b.x, a.y - b.y}; }
 __device__ __forceinline__ double2 pmul(double2 a, double2 b) { return double2{a.x * b.x, a.y * b.y}; }
 
+// (double)f on the integer pipe: GB300's FP64 pipe, which also converts, takes 16 cycles a
+// warp instruction per SM.  Exact; subnormals, infinities and NaN take the conversion.
+__device__ __forceinline__ double widen(float f) {
+  const unsigned u = __float_as_uint(f);
+  if (((u >> 23) & 255u) - 1u < 254u)
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+  return (u << 1) == 0u ? __hiloint2double((int)u, 0) : (double)f;
+}
+__device__ __forceinline__ double widen(double f) { return f; }
+
 // ------------------------------------------------------------------ handles
 struct Scratch {
   void* ptr = nullptr;
@@ -212,9 +222,16 @@ inline TwLayout tw_layout(int R, int C) {
 }
 
 // ---- launchers implemented in tod.cu
-int launch_map_to_gather(cmm_op* op, const double* m);
+int launch_map_to_gather(cmm_op* op, const double* m, bool clear_acc);
 int launch_acc_to_map(cmm_op* op, double* out);
-int launch_apply_chunk(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, int pass = -1);
+// Whether the last binning launch of an application writes the result itself, and whether
+// the FP64 accumulator takes part (else it needs no clearing).
+bool apply_direct(const cmm_op* op);
+bool apply_uses_acc(const cmm_op* op);
+// out: the result map, which the last chunk of a direct application writes (else unused)
+int launch_apply_chunk(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, double* out, int pass = -1);
+// out = P^T N^-1 P m, or P^T N^-1 tod where tod is given
+int launch_apply(cmm_op* op, const double* m, const void* tod, int tod_is_f64, double* out);
 int launch_project(cmm_op* op, const double* m, void* tod, int tod_is_f64);
 int launch_hit_blocks(cmm_pointing* pt, const double* det_weight, const uint8_t* mask, double* blocks);
 int op_init_twiddles(cmm_op* op);
@@ -228,7 +245,7 @@ bool fast_path_sizes(int logN, int prec, int* logR, int* logC);
 bool pair_path_fits(const cmm_op* op);
 bool pair_path_ok(const cmm_op* op);
 bool pair_path_sizes(int log_nt, int* logR, int* logC);
-int launch_apply_chunk_pair(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, int pass);
+int launch_apply_chunk_pair(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, double* out, int pass);
 int launch_apply_chunk_pair64(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, int pass);
 int prepare_pair(cmm_op* op);
 int prepare_pair64(cmm_op* op);

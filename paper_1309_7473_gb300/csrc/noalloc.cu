@@ -85,14 +85,9 @@ int cmm_apply_A_noalloc(cmm_op* op, const double* m_in, double* m_out) {
   }
 
   // The array keeps whatever the previous call left: the FP32 partial map must
-  // start at zero (the FP64 accumulator is cleared by the gather kernel).
+  // start at zero (the FP64 accumulator is cleared with the gather copy where it is used).
   CMM_CUDA(cudaMemsetAsync(v.acc32, 0, sizeof(float) * op->acc_stride * (npix + 1), op->ctx->stream));
-  CMM_TRY(launch_map_to_gather(&v, m_in));
-  for (int d0 = 0; d0 < op->pt->n_det; d0 += v.chunk) {
-    const int nd = std::min(v.chunk, op->pt->n_det - d0);
-    CMM_TRY(launch_apply_chunk(&v, d0, nd, nullptr, 0));
-  }
-  return launch_acc_to_map(&v, m_out);
+  return launch_apply(&v, m_in, nullptr, 0, m_out);
 }
 
 }  // extern "C"

@@ -398,19 +398,20 @@ int op_init_twiddles(cmm_op* op) {
 }
 
 template <typename T, int NC>
-static int map_to_gather_t(cmm_op* op, const double* m) {
+static int map_to_gather_t(cmm_op* op, const double* m, bool clear_acc) {
   const long long npix = op->pt->npix;
   const int blocks = (int)std::min<long long>((npix + 255) / 256, 4096);
   k_map_to_gather<T, NC><<<blocks, 256, 0, op->ctx->stream>>>(m, op->pt->mask, op->gather, op->acc,
-                                                              op->acc_stride, npix, op->done);
+                                                              clear_acc ? op->acc_stride : 0, npix, op->done);
   CMM_LAUNCH_CHECK();
   return CMM_OK;
 }
 
-int launch_map_to_gather(cmm_op* op, const double* m) {
+int launch_map_to_gather(cmm_op* op, const double* m, bool clear_acc) {
   const bool f64 = op->prec == CMM_PREC_F64;
-  if (op->pt->ncomp == 1) return f64 ? map_to_gather_t<double, 1>(op, m) : map_to_gather_t<float, 1>(op, m);
-  return f64 ? map_to_gather_t<double, 3>(op, m) : map_to_gather_t<float, 3>(op, m);
+  if (op->pt->ncomp == 1)
+    return f64 ? map_to_gather_t<double, 1>(op, m, clear_acc) : map_to_gather_t<float, 1>(op, m, clear_acc);
+  return f64 ? map_to_gather_t<double, 3>(op, m, clear_acc) : map_to_gather_t<float, 3>(op, m, clear_acc);
 }
 
 int launch_acc_to_map(cmm_op* op, double* out) {
@@ -487,9 +488,9 @@ static int apply_chunk_nc(cmm_op* op, int d0, int nd, const void* tod, int pass)
   }
 }
 
-int launch_apply_chunk(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, int pass) {
+int launch_apply_chunk(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, double* out, int pass) {
   const int nc = op->pt->ncomp;
-  if (pair_path_ok(op)) return launch_apply_chunk_pair(op, d0, nd, tod, tod_is_f64, pass);
+  if (pair_path_ok(op)) return launch_apply_chunk_pair(op, d0, nd, tod, tod_is_f64, out, pass);
   if (fast_path_ok(op)) {
     if (op->pt->max_hits <= kF32HitLimit || pass == 0 || pass == 1)
       return launch_apply_chunk_fast(op, d0, nd, tod, tod_is_f64, pass);
@@ -504,6 +505,26 @@ int launch_apply_chunk(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f
   if (!tod) return nc == 1 ? apply_chunk_nc<1, 0>(op, d0, nd, nullptr, pass) : apply_chunk_nc<3, 0>(op, d0, nd, nullptr, pass);
   if (tod_is_f64) return nc == 1 ? apply_chunk_nc<1, 2>(op, d0, nd, tod, pass) : apply_chunk_nc<3, 2>(op, d0, nd, tod, pass);
   return nc == 1 ? apply_chunk_nc<1, 1>(op, d0, nd, tod, pass) : apply_chunk_nc<3, 1>(op, d0, nd, tod, pass);
+}
+
+// The FP32 binning sums one partial map per group of detectors; its last flush can write
+// the result, so that the FP64 accumulator only serves applications of several flushes.
+bool apply_direct(const cmm_op* op) { return pair_path_ok(op) && op->prec != CMM_PREC_F64; }
+
+bool apply_uses_acc(const cmm_op* op) {
+  return !apply_direct(op) || op->chunk < op->pt->n_det || op->pt->n_det > op->acc32_maps * kFlushDets;
+}
+
+int launch_apply(cmm_op* op, const double* m, const void* tod, int tod_is_f64, double* out) {
+  const bool acc = apply_uses_acc(op);
+  if (!tod) CMM_TRY(launch_map_to_gather(op, m, acc));
+  else if (acc)
+    CMM_CUDA(cudaMemsetAsync(op->acc, 0, sizeof(double) * op->acc_stride * op->pt->npix, op->ctx->stream));
+  for (int d0 = 0; d0 < op->pt->n_det; d0 += op->chunk) {
+    const int nd = std::min(op->chunk, op->pt->n_det - d0);
+    CMM_TRY(launch_apply_chunk(op, d0, nd, tod, tod_is_f64, out));
+  }
+  return apply_direct(op) ? CMM_OK : launch_acc_to_map(op, out);
 }
 
 int launch_generic_fwd_from_tod(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64) {
@@ -530,7 +551,7 @@ static int project_t(cmm_op* op, void* tod, int tod_is_f64) {
 }
 
 int launch_project(cmm_op* op, const double* m, void* tod, int tod_is_f64) {
-  CMM_TRY(launch_map_to_gather(op, m));
+  CMM_TRY(launch_map_to_gather(op, m, false));
   const bool f64 = op->prec == CMM_PREC_F64;
   if (op->pt->ncomp == 1) return f64 ? project_t<double, 1>(op, tod, tod_is_f64) : project_t<float, 1>(op, tod, tod_is_f64);
   return f64 ? project_t<double, 3>(op, tod, tod_is_f64) : project_t<float, 3>(op, tod, tod_is_f64);

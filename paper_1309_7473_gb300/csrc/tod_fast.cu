@@ -524,16 +524,16 @@ __global__ void k_fast_flush(float* __restrict__ acc32, double* __restrict__ acc
     if (NC == 1) {
       const float v = acc32[p];
       if (v != 0.0f) {
-        acc[p] += (double)v;
+        acc[p] += widen(v);
         acc32[p] = 0.0f;
       }
     } else {
       const float4 v = reinterpret_cast<float4*>(acc32)[p];
       if (v.x != 0.0f || v.y != 0.0f || v.z != 0.0f) {
         double* o = acc + 4 * p;
-        o[0] += (double)v.x;
-        o[1] += (double)v.y;
-        o[2] += (double)v.z;
+        o[0] += widen(v.x);
+        o[1] += widen(v.y);
+        o[2] += widen(v.z);
         reinterpret_cast<float4*>(acc32)[p] = make_float4(0.f, 0.f, 0.f, 0.f);
       }
     }
@@ -673,7 +673,7 @@ __global__ void k_fast_flush_maps(float* __restrict__ acc32, int maps, long long
         float* q = acc32 + g * map_elems + p;
         const float v = *q;
         if (v != 0.0f) {
-          s += (double)v;
+          s += widen(v);
           *q = 0.0f;
           any = true;
         }
@@ -686,9 +686,9 @@ __global__ void k_fast_flush_maps(float* __restrict__ acc32, int maps, long long
         float4* q = reinterpret_cast<float4*>(acc32 + g * map_elems) + p;
         const float4 v = *q;
         if (v.x != 0.0f || v.y != 0.0f || v.z != 0.0f) {
-          s0 += (double)v.x;
-          s1 += (double)v.y;
-          s2 += (double)v.z;
+          s0 += widen(v.x);
+          s1 += widen(v.y);
+          s2 += widen(v.z);
           *q = make_float4(0.f, 0.f, 0.f, 0.f);
           any = true;
         }
@@ -701,6 +701,64 @@ __global__ void k_fast_flush_maps(float* __restrict__ acc32, int maps, long long
       }
     }
   }
+}
+
+// The last flush of an application: out = (accumulator +) the sum of the partial maps in
+// FP64, zero on masked pixels, and the partial maps cleared.  With one flush an
+// application (the usual case) this replaces the accumulator's clearing, its update and
+// its copy: 75 -> 38 us of an application at 1024 x 2^20 on 1200 x 900 TQU, 12.4 -> 8 us
+// of the map side and one launch in six at 64 x 64.
+template <int NC>
+__global__ void k_flush_to_map(float* __restrict__ acc32, int maps, long long map_elems, const double* __restrict__ acc,
+                               const uint8_t* __restrict__ mask, double* __restrict__ out, long long npix,
+                               const int* done) {
+  if (done && *done) return;
+  for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < npix;
+       p += (long long)gridDim.x * blockDim.x) {
+    const bool ok = mask[p] != 0;
+    if (NC == 1) {
+      double s = acc ? acc[p] : 0.0;
+      for (int g = 0; g < maps; ++g) {
+        float* q = acc32 + g * map_elems + p;
+        const float v = *q;
+        if (v != 0.0f) {
+          s += widen(v);
+          *q = 0.0f;
+        }
+      }
+      out[p] = ok ? s : 0.0;
+    } else {
+      double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+      if (acc) {
+        s0 = acc[4 * p];
+        s1 = acc[4 * p + 1];
+        s2 = acc[4 * p + 2];
+      }
+      for (int g = 0; g < maps; ++g) {
+        float4* q = reinterpret_cast<float4*>(acc32 + g * map_elems) + p;
+        const float4 v = *q;
+        if (v.x != 0.0f || v.y != 0.0f || v.z != 0.0f) {
+          s0 += widen(v.x);
+          s1 += widen(v.y);
+          s2 += widen(v.z);
+          *q = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+      }
+      out[p] = ok ? s0 : 0.0;
+      out[npix + p] = ok ? s1 : 0.0;
+      out[2 * npix + p] = ok ? s2 : 0.0;
+    }
+  }
+}
+
+int launch_flush_to_map(const TodArgs& a, int nc, int maps, bool add_acc, const uint8_t* mask, double* out,
+                        cudaStream_t st) {
+  const int blocks = (int)std::min<long long>((a.npix + 255) / 256, 4096);
+  const double* acc = add_acc ? a.acc : nullptr;
+  if (nc == 1) k_flush_to_map<1><<<blocks, 256, 0, st>>>(a.acc32, maps, a.acc32_map, acc, mask, out, a.npix, a.done);
+  else k_flush_to_map<3><<<blocks, 256, 0, st>>>(a.acc32, maps, a.acc32_map, acc, mask, out, a.npix, a.done);
+  CMM_LAUNCH_CHECK();
+  return CMM_OK;
 }
 
 int launch_flush(const TodArgs& a, int nc, cudaStream_t st);

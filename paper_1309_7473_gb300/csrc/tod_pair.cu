@@ -22,11 +22,12 @@ bool pair_path_fits(const cmm_op* op) {
 
 bool pair_path_ok(const cmm_op* op) { return op->pair && pair_path_fits(op); }
 
-int launch_flush(const TodArgs& a, int nc, cudaStream_t st);
+int launch_flush_to_map(const TodArgs& a, int nc, int maps, bool add_acc, const uint8_t* mask, double* out,
+                        cudaStream_t st);
 int launch_flush_maps(const TodArgs& a, int nc, int maps, cudaStream_t st);
 
 template <typename S>
-static int apply_pair_s(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, int pass) {
+static int apply_pair_s(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, double* out, int pass) {
   TodArgs a = pair_args(op, d0);
   a.tod = tod;
   cudaStream_t st = op->ctx->stream;
@@ -43,8 +44,10 @@ static int apply_pair_s(cmm_op* op, int d0, int nd, const void* tod, int tod_is_
   }
   if (pass < 0 || pass == 2) {
     TraceRange tr("A: inverse column FFTs + P^T");
-    // one launch bins up to acc32_maps groups of kFlushDets detectors, each group
-    // into its own FP32 partial map; one flush then adds them all into FP64
+    // one launch bins up to acc32_maps groups of kFlushDets detectors, each group into its
+    // own FP32 partial map; one flush then adds them all in FP64 into the accumulator, the
+    // application's last one into the result
+    const bool acc = apply_uses_acc(op);
     const int per_launch = op->acc32_maps * kFlushDets;   // even: whole pairs per group
     for (int g0 = 0; g0 < nd; g0 += per_launch) {
       TodArgs b = a;
@@ -55,17 +58,19 @@ static int apply_pair_s(cmm_op* op, int d0, int nd, const void* tod, int tod_is_
       b.acc32_map = (long long)op->acc_stride * (a.npix + 1);
       if (nc == 1) CMM_TRY((dispatch_pair_T<float, 1, S>(b, gn, 2, st, false)));
       else CMM_TRY((dispatch_pair_T<float, 3, S>(b, gn, 2, st, false)));
-      CMM_TRY(launch_flush_maps(b, nc, (gn + kFlushDets - 1) / kFlushDets, st));
+      const int maps = (gn + kFlushDets - 1) / kFlushDets;
+      if (d0 + g0 + gn == op->pt->n_det) CMM_TRY(launch_flush_to_map(b, nc, maps, acc, op->pt->mask, out, st));
+      else CMM_TRY(launch_flush_maps(b, nc, maps, st));
     }
   }
   return CMM_OK;
 }
 
 // tod: stored data [n_det][n_t] in place of P m, or nullptr.
-int launch_apply_chunk_pair(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, int pass) {
+int launch_apply_chunk_pair(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, double* out, int pass) {
   if (op->prec == CMM_PREC_F64) return launch_apply_chunk_pair64(op, d0, nd, tod, tod_is_f64, pass);
-  if (op->prec == CMM_PREC_BF16) return apply_pair_s<__nv_bfloat162>(op, d0, nd, tod, tod_is_f64, pass);
-  return apply_pair_s<float2>(op, d0, nd, tod, tod_is_f64, pass);
+  if (op->prec == CMM_PREC_BF16) return apply_pair_s<__nv_bfloat162>(op, d0, nd, tod, tod_is_f64, out, pass);
+  return apply_pair_s<float2>(op, d0, nd, tod, tod_is_f64, out, pass);
 }
 
 // The split, which n_samp fixes, its tables and the kernels' shared-memory attributes.
