@@ -18,9 +18,9 @@
 // passes (900 = 9 10 10, 1200 = 12 10 10), the first reading global memory and the last
 // writing it.  Against one kernel per step (seven, with
 // double-buffered passes of radix 2 to 5, five for 900 and 1200) the planes cross L2
-// four times instead of ten: one apply at 1200 x 900 FP32 154 -> 62 us (rows 16, columns
-// 23, rows 17; 117 MB of maps and blocks: 17 us of HBM), 600 x 450 33 us, 256 x 256 54 -> 24,
-// 64 x 64 35 -> 23 (FP64 59 -> 45).  What bounds it now is latency at 24 warps per SM, and
+// four times instead of ten: one apply at 1200 x 900 FP32 154 -> 66 us (rows 17, columns
+// 24, rows 19; 117 MB of maps and blocks: 17 us of HBM), 600 x 450 33 us, 256 x 256 54 -> 26,
+// 64 x 64 35 -> 23 (FP64 59 -> 42).  What bounds it now is latency at 24 warps per SM, and
 // in the last kernel the FP64 pipe (z and its product with r).
 #include <math.h>
 
@@ -146,7 +146,7 @@ __device__ __forceinline__ void cx_dft_n(Cx2<T>* x) {
 // Launch shapes.  FP32: at most 12 points a thread (48 registers of data), two columns
 // beside each other to make whole 32-byte sectors, and registers for three row blocks and
 // two column blocks per SM (two and one: 84 against 62 us an apply at 1200 x 900, four row
-// blocks 64).  FP64: at most 6 points, since its pipe takes as long for a warp with few
+// blocks 64, with twiddles formed in registers).  FP64: at most 6 points, since its pipe takes as long for a warp with few
 // lanes as for a full one, so small maps want many threads a line (64 x 64: 45 us an apply
 // in radix 4, 76 in radix 8).
 template <typename T> struct CircKernel {
@@ -159,8 +159,9 @@ template <typename T> struct CircKernel {
 // Inputs i + m nbf of one butterfly, from load(pos) or from buf (positions through
 // at(pos)), its stage twiddles (for a pass after the first) and its transform.
 template <typename T, int SIGN, int R, typename At, typename Load>
-__device__ __forceinline__ void butterfly_in(Cx2<T> (&x)[CircKernel<T>::kMaxRad], int i, int nbf, bool rd, bool twiddle, const V2<T>* tw,
-                                             const Cx2<T>* buf, const At& at, const Load& load) {
+__device__ __forceinline__ void butterfly_in(Cx2<T> (&x)[CircKernel<T>::kMaxRad], int i, int nbf, bool rd, bool twiddle,
+                                             const V2<T>* tw, int step, const Cx2<T>* buf, const At& at,
+                                             const Load& load) {
   if (rd) {
 #pragma unroll
     for (int m = 0; m < R; ++m) x[m] = buf[at(i + m * nbf)];
@@ -169,15 +170,12 @@ __device__ __forceinline__ void butterfly_in(Cx2<T> (&x)[CircKernel<T>::kMaxRad]
     for (int m = 0; m < R; ++m) x[m] = load(i + m * nbf);
   }
   if (twiddle) {
-    // powers of one loaded w, formed in four chains
-    V2<T> w = *tw;
-    if (SIGN > 0) w.y = -w.y;
-    const V2<T> w2 = cmul(w, w), w4 = cmul(w2, w2);
-    V2<T> wq[4] = {w, w2, cmul(w2, w), w4};
+    // w^m from the table: powers formed in registers lose digits (an apply at 1200 x 900 is 62
+    // us with them instead of 66, but 3e-7 from the line FFTs instead of 1.5e-7)
 #pragma unroll
     for (int m = 1; m < R; ++m) {
-      x[m] = cx_mul<T>(x[m], wq[(m - 1) & 3].x, wq[(m - 1) & 3].y);
-      if (m + 4 < R) wq[(m - 1) & 3] = cmul(wq[(m - 1) & 3], w4);
+      const V2<T> w = __ldg(tw + m * step);
+      x[m] = cx_mul<T>(x[m], w.x, SIGN > 0 ? -w.y : w.y);
     }
   }
   cx_dft_n<T, R, SIGN>(x);
@@ -235,7 +233,7 @@ __device__ __forceinline__ void line_fft(const CircLine& ln, const V2<T>* __rest
     Cx2<T> x[CircKernel<T>::kMaxRad];
     if (act)
       for_radix<T>(R, [&](auto r) {
-        butterfly_in<T, SIGN, decltype(r)::value>(x, i, nbf, rd, st > 0, tw + k * ln.step[st], buf, at, load);
+        butterfly_in<T, SIGN, decltype(r)::value>(x, i, nbf, rd, st > 0, tw, k * ln.step[st], buf, at, load);
       });
     if (rd && wr) __syncthreads();   // every input of this pass has been read
     if (act)
