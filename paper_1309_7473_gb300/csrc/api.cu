@@ -598,11 +598,17 @@ int cmm_op_set_pixel_cache(cmm_op* op, int32_t enable) {
   return s;
 }
 
+// The packing in use; the correlated-noise tables are in the slot order of one of them.
+static void set_pair(cmm_op* op, int pair) {
+  if (op->pair != pair && op->nz->corr_r > 0) op->corr_version = -1;
+  op->pair = pair;
+}
+
 int cmm_op_set_pair_packing(cmm_op* op, int32_t enable) {
   if (!op) return fail(CMM_ERR_ARG, "null argument");
   CMM_CUDA(cudaSetDevice(op->ctx->device));
   CMM_CUDA(cudaStreamSynchronize(op->ctx->stream));
-  op->pair = enable ? 1 : 0;
+  set_pair(op, enable ? 1 : 0);
   return CMM_OK;
 }
 
@@ -625,8 +631,9 @@ int op_sync_corr(cmm_op* op) {
     if (op->chunk < op->pt->n_det)
       return fail(CMM_ERR_UNSUPPORTED, "correlated noise needs every detector in one chunk (det_chunk)");
     const int r = nz->corr_r;
-    CMM_TRY(dalloc(&op->corr_minv, sizeof(float) * (size_t)(op->N + 1) * r * r));
-    CMM_TRY(dalloc(&op->corr_s, sizeof(float2) * (size_t)op->N * r));
+    const size_t slots = pair_path_ok(op) ? (size_t)pair_corr_slots_of(op) : (size_t)op->N + 1;
+    CMM_TRY(dalloc(&op->corr_minv, sizeof(float) * slots * r * r));
+    CMM_TRY(dalloc(&op->corr_s, sizeof(float2) * slots * r));
     CMM_TRY(launch_corr_minv(op, nz->corr_par, op->corr_minv));
     CMM_CUDA(cudaStreamSynchronize(op->ctx->stream));
   }
@@ -1476,10 +1483,10 @@ std::vector<std::pair<TuneKey, int>> g_tune_cache;
 // (its split is fixed by n_samp), lr > 0 = one-detector packing with R = 2^lr.
 static int apply_decision(cmm_op* op, int v) {
   if (v == 0) {
-    op->pair = 1;
+    set_pair(op, 1);
     return CMM_OK;
   }
-  op->pair = 0;
+  set_pair(op, 0);
   return v != op->logR ? op_set_split(op, v) : CMM_OK;
 }
 
@@ -1494,7 +1501,7 @@ int cmm_autotune(cmm_op* op, int32_t reps, const char* cache_path, int32_t* chos
   CMM_CUDA(cudaSetDevice(op->ctx->device));
   const TuneKey key{op->pt->n_t, op->pt->n_det, op->prec, op->pt->ncomp};
   const int logN = op->logR + op->logC;
-  const bool pair_ok = pair_path_fits(op);
+  const bool pair_ok = pair_path_fits(op) && op->nz->corr_r == 0;
   auto valid = [&](int v) { return (v == 0 && pair_ok) || (v > 0 && v < logN); };
   // cached decision (process-wide, then the optional file)
   for (auto& e : g_tune_cache)

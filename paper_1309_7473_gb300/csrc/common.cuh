@@ -186,8 +186,8 @@ struct cmm_op {
   double2* rot64 = nullptr;    // FP64 two-detector path: [n_t] (cos 2phi, sin 2phi)
   double* lg2 = nullptr;       // the same: [n_t / 2 + 1] log2 of the frequency index, 64 powers 2^(j / 64)
   int corr_version = 0;        // noise correlation version the tables below were built for
-  float* corr_minv = nullptr;  // [N + 1][r][r] per-bin M^-1 in slot order (index N: bin N)
-  float2* corr_s = nullptr;    // [N][r] cross-detector solution per bin slot
+  float* corr_minv = nullptr;  // per-bin M^-1, [r][r] each, in the slot order of the path in use
+  float2* corr_s = nullptr;    // cross-detector solution per bin slot ([slots][r], two-detector path [r][slots])
   double* tmp_a = nullptr;     // [ncomp*npix] device temporaries
   double* tmp_b = nullptr;
   const int* done = nullptr;   // solver stop flag seen by every kernel (nullptr: none)
@@ -244,6 +244,7 @@ bool fast_path_sizes(int logN, int prec, int* logR, int* logC);
 // ---- two-detector path (tod_pair.cu, its FP64 form in tod_pair64.cu)
 bool pair_path_fits(const cmm_op* op);
 bool pair_path_ok(const cmm_op* op);
+int pair_corr_slots_of(const cmm_op* op);   // bin slots of the correlated-noise tables
 bool pair_path_sizes(int log_nt, int* logR, int* logC);
 int launch_apply_chunk_pair(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, double* out, int pass);
 int launch_apply_chunk_pair64(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, int pass);

@@ -37,7 +37,7 @@ namespace cmm {
 
 // w_d(f_k): the detector's tabulated weight when the noise has a table, else the law
 __device__ __forceinline__ float filter_weight_fast(const TodArgs& a, int d, const float4 cf, int k) {
-  if (a.wtab) return __ldg(reinterpret_cast<const float*>(a.wtab) + (size_t)d * (a.N + 1) + k);
+  if (a.wtab) return __ldg(reinterpret_cast<const float*>(a.wtab) + (size_t)d * (a.n_t / 2 + 1) + k);
   return filter_weight_law(cf, k);
 }
 
@@ -349,15 +349,18 @@ __global__ void k_fast_corr(const TodArgs a, int n_det) {
   }
 }
 
-// M(k)^-1 per bin slot (slot order of the op's split; index N: bin N):
+// M(k)^-1 per bin slot, in the order of the one-detector split (index N: bin N) or, with
+// pair_slots, of the two-detector path's (slot k1 C + pos: bin k1 + R pos or its mirror):
 // M = diag(1 / e_j(k)) + sum_d w_d(k) V_d V_d^T, accumulated and inverted in FP64
 // (Gauss-Jordan with partial pivoting, r <= 4), stored in FP32.
 __global__ void k_corr_minv(const TodArgs a, int n_det, const double* __restrict__ mode_par, double f_samp,
-                            float* __restrict__ minv) {
+                            float* __restrict__ minv, int slots, bool pair_slots) {
   const int slot = blockIdx.x * blockDim.x + threadIdx.x;
-  if (slot > a.N) return;
+  if (slot >= slots) return;
   const int r = a.corr_r;
-  const int k = slot == (int)a.N ? (int)a.N : (slot & (a.C - 1)) * a.R + (slot >> a.logC);
+  int k = (slot & (a.C - 1)) * a.R + (slot >> a.logC);
+  if (pair_slots) k = min(k, (int)a.n_t - k);
+  else if (slot == (int)a.N) k = (int)a.N;
   double m[kMaxCorrModes][2 * kMaxCorrModes];
   const double f = (double)(k == 0 ? 1 : k) * f_samp / (double)a.n_t;
   for (int j = 0; j < r; ++j) {
@@ -838,9 +841,15 @@ static int prepare_fast_s(cmm_op* op) {
 int launch_corr_minv(cmm_op* op, const double* mode_par_dev, float* minv) {
   TodArgs a = make_args(op, 0);
   a.corr_r = op->nz->corr_r;   // the tables are being built: make_args does not count them yet
-  const long long n = op->N + 1;
-  k_corr_minv<<<(int)((n + 127) / 128), 128, 0, op->ctx->stream>>>(a, op->pt->n_det, mode_par_dev, op->nz->f_samp,
-                                                                  minv);
+  const bool pair = pair_path_ok(op);
+  if (pair) {
+    a.R = op->pR;
+    a.C = op->pC;
+    a.logC = op->plogC;
+  }
+  const int n = pair ? pair_corr_slots_of(op) : (int)op->N + 1;
+  k_corr_minv<<<(n + 127) / 128, 128, 0, op->ctx->stream>>>(a, op->pt->n_det, mode_par_dev, op->nz->f_samp, minv, n,
+                                                           pair);
   CMM_LAUNCH_CHECK();
   return CMM_OK;
 }

@@ -14,17 +14,33 @@ bool pair_path_sizes(int log_nt, int* logR, int* logC) {
 }
 
 // Whether the path can serve the operator's applications (the hit limit is that of the
-// FP32 partial maps), and whether it does.
+// FP32 partial maps; correlated noise is for FP32 and BF16), and whether it does.
 bool pair_path_fits(const cmm_op* op) {
-  return op->pR > 0 && op->tw_pair && op->nz->corr_r == 0 &&
-         (op->prec == CMM_PREC_F64 || op->pt->max_hits <= kF32HitLimit);
+  return op->pR > 0 && op->tw_pair &&
+         (op->prec == CMM_PREC_F64 ? op->nz->corr_r == 0 : op->pt->max_hits <= kF32HitLimit);
 }
+
+int pair_corr_slots_of(const cmm_op* op) { return pair_corr_slots(op->pR, op->pC); }
 
 bool pair_path_ok(const cmm_op* op) { return op->pair && pair_path_fits(op); }
 
 int launch_flush_to_map(const TodArgs& a, int nc, int maps, bool add_acc, const uint8_t* mask, double* out,
                         cudaStream_t st);
 int launch_flush_maps(const TodArgs& a, int nc, int maps, cudaStream_t st);
+
+template <typename S>
+static int run_corr(const TodArgs& a, int nd, cudaStream_t st) {
+  const int g = (pair_corr_slots(a.R, a.C) + kCorrThreads - 1) / kCorrThreads;
+  switch (a.corr_r) {
+    case 1: k_pair_corr<S, 1><<<g, kCorrThreads, 0, st>>>(a, nd); break;
+    case 2: k_pair_corr<S, 2><<<g, kCorrThreads, 0, st>>>(a, nd); break;
+    case 3: k_pair_corr<S, 3><<<g, kCorrThreads, 0, st>>>(a, nd); break;
+    default: k_pair_corr<S, 4><<<g, kCorrThreads, 0, st>>>(a, nd); break;
+  }
+  CMM_LAUNCH_CHECK();
+  return CMM_OK;
+}
+static_assert(kMaxCorrModes == 4, "k_pair_corr instances");
 
 template <typename S>
 static int apply_pair_s(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, double* out, int pass) {
@@ -40,7 +56,14 @@ static int apply_pair_s(cmm_op* op, int d0, int nd, const void* tod, int tod_is_
   }
   if (pass < 0 || pass == 1) {
     TraceRange tr("A: row FFTs + N^-1");
-    CMM_TRY((dispatch_pair_F<float, S>(a, nd, st, false)));
+    if (a.corr_r > 0) {
+      // correlated noise: forward rows, the cross-detector solve over the whole chunk, back
+      CMM_TRY((dispatch_pair_F<float, S, kPairSplit>(a, nd, st, false)));
+      CMM_TRY(run_corr<S>(a, nd, st));
+      CMM_TRY((dispatch_pair_F<float, S, kPairMerge>(a, nd, st, false)));
+    } else {
+      CMM_TRY((dispatch_pair_F<float, S>(a, nd, st, false)));
+    }
   }
   if (pass < 0 || pass == 2) {
     TraceRange tr("A: inverse column FFTs + P^T");

@@ -124,19 +124,29 @@ __device__ __forceinline__ float pair_weight(const TodArgs& a, int d, const floa
   return filter_weight_law(cf, kf);
 }
 
-// The pair filter's a, b = (w_d1 +- w_d2) / 2 at frequency index kf: from the tables, else
-// the law with log2(kf) shared
-__device__ __forceinline__ void pair_ab(const TodArgs& a, int d1, int d2, const float4 cf1, const float4 cf2, bool two,
-                                        int kf, float& ha, float& hb) {
-  float w1, w2;
+// w of one detector from log2 of its frequency index
+__device__ __forceinline__ float law_weight(const float4 cf, float lk) {
+  return cf.w != 0.0f ? cf.x : __fdividef(cf.x, 1.0f + exp2f(fmaf(-cf.y, lk, cf.z)));
+}
+
+// w_d1 and w_d2 at frequency index kf: from the tables, else the law with log2(kf) shared
+__device__ __forceinline__ void pair_weights(const TodArgs& a, int d1, int d2, const float4 cf1, const float4 cf2,
+                                             bool two, int kf, float& w1, float& w2) {
   if (a.wtab) {
     w1 = pair_weight(a, d1, cf1, kf);
     w2 = two ? pair_weight(a, d2, cf2, kf) : 0.f;
   } else {
     const float lk = __log2f(small_int_to_float(kf == 0 ? 1 : kf));
-    w1 = cf1.w != 0.0f ? cf1.x : __fdividef(cf1.x, 1.0f + exp2f(fmaf(-cf1.y, lk, cf1.z)));
-    w2 = !two ? 0.f : cf2.w != 0.0f ? cf2.x : __fdividef(cf2.x, 1.0f + exp2f(fmaf(-cf2.y, lk, cf2.z)));
+    w1 = law_weight(cf1, lk);
+    w2 = two ? law_weight(cf2, lk) : 0.f;
   }
+}
+
+// The pair filter's a, b = (w_d1 +- w_d2) / 2
+__device__ __forceinline__ void pair_ab(const TodArgs& a, int d1, int d2, const float4 cf1, const float4 cf2, bool two,
+                                        int kf, float& ha, float& hb) {
+  float w1, w2;
+  pair_weights(a, d1, d2, cf1, cf2, two, kf, w1, w2);
   ha = 0.5f * (w1 + w2);
   hb = 0.5f * (w1 - w2);
 }
@@ -331,7 +341,19 @@ template <typename T, int C, int E> struct PairFilterShape {
   static constexpr int MINB = sizeof(T) == 8 ? 1 : 512 / THREADS;
 };
 
-template <typename T, typename S, int E, int... RC>
+// The spectrum slots of the cross-detector step: slot k1 C + pos holds bin k = k1 + R pos,
+// k1 = 0 .. R / 2 (rows 0 and R / 2 hold every bin twice, conjugated).
+__host__ __device__ __forceinline__ int pair_corr_slots(int R, int C) { return (R / 2 + 1) * C; }
+
+// Modes.  kPairFull: the whole pass.  With noise correlated between detectors the pass is
+// cut around k_pair_corr: kPairSplit stores the forward transforms, Z(k) in row k1 and
+// conj Z(n - k) in row R - k1 (rows 0 and R / 2: Z(k) alone, whose partner is in the same
+// row); kPairMerge starts from those, y_j = w_j (S_j - sum_m V_jm s_m) with the spectra
+// S_1 = (A + B) / 2 and S_2 = (A - B) / 2i of the two detectors, and inverts
+// (A, B) = (y_1 + i y_2, y_1 - i y_2).
+constexpr int kPairFull = 0, kPairSplit = 1, kPairMerge = 2;
+
+template <typename T, typename S, int MODE, int E, int... RC>
 __global__ void __launch_bounds__(PairFilterShape<T, RadProd<RC...>::value, E>::THREADS,
                                   PairFilterShape<T, RadProd<RC...>::value, E>::MINB)
     k_pair_filter(const TodArgs a, int nd) {
@@ -356,41 +378,98 @@ __global__ void __launch_bounds__(PairFilterShape<T, RadProd<RC...>::value, E>::
   S* Yb = lo ? Ya : Ya + (a.R - 2 * k1) * C;   // row R - k1
   const RowAddr2<T, PS> ad{reinterpret_cast<Cx2<T>*>(smraw) + rs * ROWLEN};
   Cx2<T> x[E];
+  if constexpr (MODE == kPairMerge) {
+    if (lo || mid) {   // the partner position of the same row, conjugated
+      const S* row = Ya - i;
 #pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const V A = ok ? Store<T, S>::ld(Ya + e * TPR) : V{(T)0, (T)0};
-    const V B = ok ? Store<T, S>::ld(Yb + e * TPR) : V{(T)0, (T)0};
-    x[e] = Cx2<T>{V{A.x, B.x}, V{A.y, B.y}};
-  }
-  if (lo) {
+      for (int e = 0; e < E; ++e) {
+        const int pos = i + e * TPR;
+        const V A = Store<T, S>::ld(row + pos), B = Store<T, S>::ld(row + (lo ? (C - pos) & (C - 1) : C - 1 - pos));
+        x[e] = Cx2<T>{V{A.x, B.x}, V{A.y, -B.y}};
+      }
+    } else {
 #pragma unroll
-    for (int e = 0; e < E; ++e) x[e].im.y = -x[e].im.x;   // B = conj A
-  } else if (mid) {
-    // row R / 2 is stored as B = conj(y) w_N^(c R / 2): A = conj(B) w_C^c
+      for (int e = 0; e < E; ++e) {
+        const V A = ok ? Store<T, S>::ld(Ya + e * TPR) : V{(T)0, (T)0};
+        const V B = ok ? Store<T, S>::ld(Yb + e * TPR) : V{(T)0, (T)0};
+        x[e] = Cx2<T>{V{A.x, B.x}, V{A.y, B.y}};
+      }
+    }
+  } else {
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-      const V A = cmul(V{x[e].re.y, -x[e].im.y}, __ldg(tw + a.twl.C_off + i + e * TPR));
-      x[e].re.x = A.x;
-      x[e].im.x = A.y;
+      const V A = ok ? Store<T, S>::ld(Ya + e * TPR) : V{(T)0, (T)0};
+      const V B = ok ? Store<T, S>::ld(Yb + e * TPR) : V{(T)0, (T)0};
+      x[e] = Cx2<T>{V{A.x, B.x}, V{A.y, B.y}};
     }
+    if (lo) {
+#pragma unroll
+      for (int e = 0; e < E; ++e) x[e].im.y = -x[e].im.x;   // B = conj A
+    } else if (mid) {
+      // row R / 2 is stored as B = conj(y) w_N^(c R / 2): A = conj(B) w_C^c
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const V A = cmul(V{x[e].re.y, -x[e].im.y}, __ldg(tw + a.twl.C_off + i + e * TPR));
+        x[e].re.x = A.x;
+        x[e].im.x = A.y;
+      }
+    }
+    rfft2<T, -1, true, E, RC...>(x, i, tw + a.twl.C_off, ad);
   }
-  rfft2<T, -1, true, E, RC...>(x, i, tw + a.twl.C_off, ad);
+  if constexpr (MODE == kPairSplit) {
+    if (ok) {
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        Store<T, S>::st(Ya + e * TPR, V{x[e].re.x, x[e].im.x});
+        if (!lo && !mid) Store<T, S>::st(Yb + e * TPR, V{x[e].re.y, x[e].im.y});
+      }
+    }
+    return;
+  }
   {
     const V4<T> cf1 = reinterpret_cast<const V4<T>*>(a.coef)[d1];
     const V4<T> cf2 = reinterpret_cast<const V4<T>*>(a.coef)[d2];
     const int n = (int)a.N;
+    float tv1[kMaxCorrModes], tv2[kMaxCorrModes];   // the detectors' templates
+    const int slots = pair_corr_slots(a.R, C);
+    if constexpr (MODE == kPairMerge) {
+#pragma unroll
+      for (int j = 0; j < kMaxCorrModes; ++j) {
+        tv1[j] = j < a.corr_r ? a.corrV[d1 * a.corr_r + j] : 0.f;
+        tv2[j] = j < a.corr_r ? a.corrV[d2 * a.corr_r + j] : 0.f;
+      }
+    }
 #pragma unroll
     for (int e = 0; e < E; ++e) {
       const int k = k1 + a.R * (i + e * TPR);
       const int kf = ok ? min(k, n - k) : 0;
-      T ha, hb;
-      pair_ab(a, d1, d2, cf1, cf2, two, kf, ha, hb);
-      const V h{ha, ha}, g{hb, hb};
-      x[e].re = pfma(h, x[e].re, pmul(g, V{x[e].re.y, x[e].re.x}));
-      x[e].im = pfma(h, x[e].im, pmul(g, V{x[e].im.y, x[e].im.x}));
+      if constexpr (MODE == kPairMerge) {
+        T w1, w2;
+        pair_weights(a, d1, d2, cf1, cf2, two, kf, w1, w2);
+        V p1{(T)0, (T)0}, p2{(T)0, (T)0};
+        const float2* sol = a.corr_s + (ok ? k1 * C + i + e * TPR : 0);
+#pragma unroll
+        for (int j = 0; j < kMaxCorrModes; ++j)
+          if (j < a.corr_r) {
+            const float2 sj = __ldg(sol + j * slots);
+            p1 = V{fmaf(tv1[j], sj.x, p1.x), fmaf(tv1[j], sj.y, p1.y)};
+            p2 = V{fmaf(tv2[j], sj.x, p2.x), fmaf(tv2[j], sj.y, p2.y)};
+          }
+        const Cx2<T> v = x[e];
+        const T h = (T)0.5;
+        const V y1{w1 * (h * (v.re.x + v.re.y) - p1.x), w1 * (h * (v.im.x + v.im.y) - p1.y)};
+        const V y2{w2 * (h * (v.im.x - v.im.y) - p2.x), w2 * (h * (v.re.y - v.re.x) - p2.y)};
+        x[e] = Cx2<T>{V{y1.x - y2.y, y1.x + y2.y}, V{y1.y + y2.x, y1.y - y2.x}};
+      } else {
+        T ha, hb;
+        pair_ab(a, d1, d2, cf1, cf2, two, kf, ha, hb);
+        const V h{ha, ha}, g{hb, hb};
+        x[e].re = pfma(h, x[e].re, pmul(g, V{x[e].re.y, x[e].re.x}));
+        x[e].im = pfma(h, x[e].im, pmul(g, V{x[e].im.y, x[e].im.x}));
+      }
     }
   }
-  rfft2<T, 1, false, E, RC...>(x, i, tw + a.twl.C_off, ad);
+  rfft2<T, 1, MODE == kPairMerge, E, RC...>(x, i, tw + a.twl.C_off, ad);
   if (ok) {
     // conj(w_N^(k1 c)), c = i + e TPR, for both rows: by recurrence, or from the tables
     V w = tw_N(a, tw, k1 * i);
@@ -403,6 +482,88 @@ __global__ void __launch_bounds__(PairFilterShape<T, RadProd<RC...>::value, E>::
       if constexpr (sizeof(T) == 4) w = cmul(w, stp);
       else if (e + 1 < E) w = tw_N(a, tw, k1 * (i + (e + 1) * TPR));
     }
+  }
+}
+
+// ------------------------------------------------------------------ correlated noise
+// Cross-detector step, one thread per slot: t_j = sum_d V_dj w_d(k) S_d(k) over all
+// detectors, s = M(k)^-1 t (see k_corr_minv).  Bound by its one read of the spectra
+// (4 bytes a sample in FP32) beside the weights; log2(k) is shared by all detectors, whose
+// coefficients and templates are staged in shared memory.  1024 x 2^20, three modes: 0.93
+// ms (4.6 TB/s) beside 1.31 ms for kPairSplit and 2.73 for kPairMerge, which reads every
+// bin's solution from L2 once per pair of detectors (8 points a thread: 2.84 ms; pairs
+// varying fastest over the blocks: 2.89).  A with three modes 13.9 -> 9.95 ms against the
+// one-detector packing, 192 x 2^19 1.39 -> 0.99.
+constexpr int kCorrThreads = 256, kCorrStage = 64;   // pairs staged at a time
+
+template <typename S, int RM>
+__global__ void __launch_bounds__(kCorrThreads) k_pair_corr(const TodArgs a, int n_det) {
+  __shared__ float4 coef[2 * kCorrStage];
+  __shared__ float V[2 * kCorrStage][RM];
+  if (a.done && *a.done) return;
+  const int slots = pair_corr_slots(a.R, a.C);
+  const int slot = min((int)(blockIdx.x * kCorrThreads + threadIdx.x), slots - 1);
+  const int k1 = slot >> a.logC, pos = slot & (a.C - 1);
+  const int k = k1 + a.R * pos, n = (int)a.N, kf = min(k, n - k);
+  const bool self = k1 == 0 || 2 * k1 == a.R;   // the partner bin in the same row
+  const int other = k1 == 0 ? ((a.C - pos) & (a.C - 1)) : self ? k1 * a.C + a.C - 1 - pos : (a.R - k1) * a.C + pos;
+  const S* Ya = reinterpret_cast<const S*>(a.spec) + slot;
+  const S* Yb = reinterpret_cast<const S*>(a.spec) + other;
+  const float lk = __log2f(small_int_to_float(kf == 0 ? 1 : kf));
+  const int pairs = (n_det + 1) / 2;
+  float2 t[RM];
+#pragma unroll
+  for (int j = 0; j < RM; ++j) t[j] = make_float2(0.f, 0.f);
+  for (int q0 = 0; q0 < pairs; q0 += kCorrStage) {
+    const int nq = min(kCorrStage, pairs - q0);
+    __syncthreads();
+    for (int d = threadIdx.x; d < 2 * nq; d += kCorrThreads) {
+      const int dd = a.d0 + min(2 * q0 + d, n_det - 1);
+      const bool real = 2 * q0 + d < n_det;   // the missing partner of an odd last detector
+      coef[d] = reinterpret_cast<const float4*>(a.coef)[dd];
+#pragma unroll
+      for (int j = 0; j < RM; ++j) V[d][j] = real ? a.corrV[dd * RM + j] : 0.f;
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int q = 0; q < nq; ++q) {
+      const size_t o = (size_t)(q0 + q) * a.N;
+      const float2 A = Store<float, S>::ld(Ya + o);
+      float2 B = Store<float, S>::ld(Yb + o);
+      if (self) B.y = -B.y;
+      float w1, w2;
+      if (a.wtab) {
+        const float* w = reinterpret_cast<const float*>(a.wtab) + kf;
+        const int d1 = a.d0 + 2 * (q0 + q);
+        w1 = __ldg(w + (size_t)d1 * (a.n_t / 2 + 1));
+        w2 = __ldg(w + (size_t)min(d1 + 1, a.d0 + n_det - 1) * (a.n_t / 2 + 1));
+      } else {
+        w1 = law_weight(coef[2 * q], lk);
+        w2 = law_weight(coef[2 * q + 1], lk);
+      }
+      w1 *= 0.5f;
+      w2 *= 0.5f;
+      const float2 s1 = make_float2(w1 * (A.x + B.x), w1 * (A.y + B.y));
+      const float2 s2 = make_float2(w2 * (A.y - B.y), w2 * (B.x - A.x));
+#pragma unroll
+      for (int j = 0; j < RM; ++j) {
+        const float v1 = V[2 * q][j], v2 = V[2 * q + 1][j];
+        t[j].x = fmaf(v1, s1.x, fmaf(v2, s2.x, t[j].x));
+        t[j].y = fmaf(v1, s1.y, fmaf(v2, s2.y, t[j].y));
+      }
+    }
+  }
+  if ((int)(blockIdx.x * kCorrThreads + threadIdx.x) >= slots) return;
+  const float* m = a.corr_minv + (size_t)slot * RM * RM;
+#pragma unroll
+  for (int j = 0; j < RM; ++j) {
+    float sx = 0.f, sy = 0.f;
+#pragma unroll
+    for (int l = 0; l < RM; ++l) {
+      sx = fmaf(m[j * RM + l], t[l].x, sx);
+      sy = fmaf(m[j * RM + l], t[l].y, sy);
+    }
+    a.corr_s[j * slots + slot] = make_float2(sx, sy);
   }
 }
 
@@ -631,45 +792,45 @@ inline int dispatch_pair_D(const TodArgs& a, int nd, bool f64, cudaStream_t st, 
   return run_pair_D<T, S, 256>(a, nd, f64, st, attr_only);
 }
 
-template <typename T, typename S, int E, int... RC>
+template <typename T, typename S, int MODE, int E, int... RC>
 inline int run_pair_F(const TodArgs& a, int nd, cudaStream_t st, bool attr_only) {
   constexpr int C = RadProd<RC...>::value;
   constexpr int PAIRS = PairFilterShape<T, C, E>::PAIRS;
   constexpr int PS = clog2(E);
   const size_t smem = sizeof(Cx2<T>) * PAIRS * (C + (C >> PS));
   if (attr_only) {
-    CMM_CUDA(cudaFuncSetAttribute(k_pair_filter<T, S, E, RC...>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CMM_CUDA(cudaFuncSetAttribute(k_pair_filter<T, S, MODE, E, RC...>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     return CMM_OK;
   }
   const int nrp = a.R / 2 + 1;
   const dim3 g((nrp + PAIRS - 1) / PAIRS, (nd + 1) / 2);
-  k_pair_filter<T, S, E, RC...><<<g, PairFilterShape<T, C, E>::THREADS, smem, st>>>(a, nd);
+  k_pair_filter<T, S, MODE, E, RC...><<<g, PairFilterShape<T, C, E>::THREADS, smem, st>>>(a, nd);
   CMM_LAUNCH_CHECK();
   return CMM_OK;
 }
 
-template <typename T, typename S>
+template <typename T, typename S, int MODE = kPairFull>
 inline int dispatch_pair_F(const TodArgs& a, int nd, cudaStream_t st, bool attr_only) {
   if constexpr (sizeof(T) == 4) {
     switch (a.logC) {
       // short rows: 8 points a thread, twice the threads (row transforms of 32 x 2^16 take
       // 10.3 against 12.4 us); from 1024 points on the third exchange costs more (75
       // against 74 us at 1024, 2.82 against 2.45 ms at 4096)
-      case 7: return run_pair_F<T, S, 8, 8, 8, 2>(a, nd, st, attr_only);
-      case 8: return run_pair_F<T, S, 8, 8, 8, 4>(a, nd, st, attr_only);
-      case 9: return run_pair_F<T, S, 8, 8, 8, 8>(a, nd, st, attr_only);
-      case 10: return run_pair_F<T, S, 16, 16, 16, 4>(a, nd, st, attr_only);
-      case 11: return run_pair_F<T, S, 16, 16, 16, 8>(a, nd, st, attr_only);
-      case 12: return run_pair_F<T, S, 16, 16, 16, 16>(a, nd, st, attr_only);
+      case 7: return run_pair_F<T, S, MODE, 8, 8, 8, 2>(a, nd, st, attr_only);
+      case 8: return run_pair_F<T, S, MODE, 8, 8, 8, 4>(a, nd, st, attr_only);
+      case 9: return run_pair_F<T, S, MODE, 8, 8, 8, 8>(a, nd, st, attr_only);
+      case 10: return run_pair_F<T, S, MODE, 16, 16, 16, 4>(a, nd, st, attr_only);
+      case 11: return run_pair_F<T, S, MODE, 16, 16, 16, 8>(a, nd, st, attr_only);
+      case 12: return run_pair_F<T, S, MODE, 16, 16, 16, 16>(a, nd, st, attr_only);
     }
   } else {
     switch (a.logC) {
-      case 7: return run_pair_F<T, S, 8, 8, 8, 2>(a, nd, st, attr_only);
-      case 8: return run_pair_F<T, S, 8, 8, 8, 4>(a, nd, st, attr_only);
-      case 9: return run_pair_F<T, S, 8, 8, 8, 8>(a, nd, st, attr_only);
-      case 10: return run_pair_F<T, S, 8, 8, 8, 8, 2>(a, nd, st, attr_only);
-      case 11: return run_pair_F<T, S, 8, 8, 8, 8, 4>(a, nd, st, attr_only);
-      case 12: return run_pair_F<T, S, 8, 8, 8, 8, 8>(a, nd, st, attr_only);
+      case 7: return run_pair_F<T, S, MODE, 8, 8, 8, 2>(a, nd, st, attr_only);
+      case 8: return run_pair_F<T, S, MODE, 8, 8, 8, 4>(a, nd, st, attr_only);
+      case 9: return run_pair_F<T, S, MODE, 8, 8, 8, 8>(a, nd, st, attr_only);
+      case 10: return run_pair_F<T, S, MODE, 8, 8, 8, 8, 2>(a, nd, st, attr_only);
+      case 11: return run_pair_F<T, S, MODE, 8, 8, 8, 8, 4>(a, nd, st, attr_only);
+      case 12: return run_pair_F<T, S, MODE, 8, 8, 8, 8, 8>(a, nd, st, attr_only);
     }
   }
   return fail(CMM_ERR_UNSUPPORTED, "pair path: row length out of range");
@@ -717,6 +878,10 @@ inline int prepare_pair_s(cmm_op* op) {
   for (const bool f64 : {false, true}) CMM_TRY((dispatch_pair_D<T, S>(a, 0, f64, nullptr, true)));
   if (op->pt->ncomp == 1) CMM_TRY((dispatch_pair_T<T, 1, S>(a, 0, 0, nullptr, true)));
   else CMM_TRY((dispatch_pair_T<T, 3, S>(a, 0, 0, nullptr, true)));
+  if constexpr (sizeof(T) == 4) {
+    CMM_TRY((dispatch_pair_F<T, S, kPairSplit>(a, 0, nullptr, true)));
+    CMM_TRY((dispatch_pair_F<T, S, kPairMerge>(a, 0, nullptr, true)));
+  }
   return dispatch_pair_F<T, S>(a, 0, nullptr, true);
 }
 
