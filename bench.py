@@ -458,7 +458,7 @@ def run_ours(args, rank, world):
     }
     # the FP32 two-detector path: the application's last flush writes the map
     map_out = 0 if args.prec != "f64" and args.corr_modes == 0 else 1
-    out["gpu_launches"] = (launches_per_iteration(scan.n_det, chunk_dets, CIRC_FUSED_LAUNCHES, map_out) * args.steps
+    out["gpu_launches"] = (launches_per_iteration(scan.n_det, chunk_dets, CIRC_FUSED_LAUNCHES, map_out, CG_FUSED_LAUNCHES) * args.steps
                            + SETUP_LAUNCHES + CIRC_FUSED_LAUNCHES)
     return out
 
@@ -655,11 +655,12 @@ def cufft_filter_ms(scan, noise, dev, stream):
                     "excludes P and P^T", "ms": ms}
 
 
-def launches_per_iteration(n_det, chunk, circ=None, map_out=1):
+def launches_per_iteration(n_det, chunk, circ=None, map_out=1, cg=None):
     """Kernels of one circulant-PCG iteration: the A-application (map copy in, per
     chunk one forward and one filter launch and, per 2048 detectors (eight FP32
     partial maps of 256 detectors), one inverse + binning launch and one flush; a map
-    copy out where the flush does not write the map), the CG update kernels and the circulant preconditioner: `circ`
+    copy out where the flush does not write the map), the `cg` update kernels (by
+    default those of the flexible solves) and the circulant preconditioner: `circ`
     kernels, by default those of the maps that the line FFTs serve (Sigma^-1,
     2-D FFTs, per-mode solve)."""
     a = 1 + map_out
@@ -667,12 +668,15 @@ def launches_per_iteration(n_det, chunk, circ=None, map_out=1):
     for d0 in range(0, n_det, chunk):
         nd = min(chunk, n_det - d0)
         a += 2 + 2 * math.ceil(nd / (256 * maps))
-    return a + CG_LAUNCHES + (CIRC_LAUNCHES if circ is None else circ)
+    return a + (CG_LAUNCHES if cg is None else cg) + (CIRC_LAUNCHES if circ is None else circ)
 
 
 # kernels per iteration outside the A-application (cmm_solve's FP64 PCG step):
 # p^T q partials, alpha, x and r update with ||r||^2, convergence check, beta, p update
 CG_LAUNCHES = 6
+# the plain FP64 PCG step: alpha with the x and r update, and the check, beta and p update
+# (p^T q comes with the application's last kernel)
+CG_FUSED_LAUNCHES = 2
 # the circulant apply: Sigma^-1 into the packed planes, 2 + 2 line-FFT passes, the
 # per-mode products, Sigma^-1 out of the planes with the r^T z partials
 CIRC_LAUNCHES = 7

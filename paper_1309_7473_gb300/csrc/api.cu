@@ -644,9 +644,10 @@ int op_sync_corr(cmm_op* op) {
 
 extern "C" {
 
-static int apply_A_dev(cmm_op* op, const double* m_in, double* m_out) {
+// With dot_partial, also the partial sums of m_in^T m_out.
+static int apply_A_dev(cmm_op* op, const double* m_in, double* m_out, double* dot_partial = nullptr) {
   TraceRange tr("cmm: A = P^T N^-1 P");
-  return launch_apply(op, m_in, nullptr, 0, m_out);
+  return launch_apply(op, m_in, nullptr, 0, ApplyOut{m_out, dot_partial ? m_in : nullptr, dot_partial});
 }
 
 int cmm_apply_A(cmm_op* op, const double* m_in, double* m_out) {
@@ -676,11 +677,11 @@ int cmm_profile_apply(cmm_op* op, const double* m_in, double* m_out, int32_t rep
       for (int d0 = 0; d0 < op->pt->n_det; d0 += op->chunk) {
         const int nd = std::min(op->chunk, op->pt->n_det - d0);
         for (int pass = 0; pass < 3; ++pass) {
-          CMM_TRY(launch_apply_chunk(op, d0, nd, nullptr, 0, m_out, pass));
+          CMM_TRY(launch_apply_chunk(op, d0, nd, nullptr, 0, ApplyOut{m_out}, pass));
           CMM_CUDA(cudaEventRecord(ev[k++], st));
         }
       }
-      if (!apply_direct(op)) CMM_TRY(launch_acc_to_map(op, m_out));
+      if (!apply_direct(op)) CMM_TRY(launch_acc_to_map(op, m_out, nullptr, nullptr));
       CMM_CUDA(cudaEventRecord(ev[k++], st));
     }
     CMM_CUDA(cudaEventRecord(ev[k++], st));
@@ -738,7 +739,7 @@ int cmm_rhs(cmm_op* op, const void* tod, int32_t tod_is_f64, double* b) {
   if (!op || !tod || !b) return fail(CMM_ERR_ARG, "null argument");
   CMM_CUDA(cudaSetDevice(op->ctx->device));
   CMM_TRY(op_sync_corr(op));
-  return launch_apply(op, nullptr, tod, tod_is_f64, b);
+  return launch_apply(op, nullptr, tod, tod_is_f64, ApplyOut{b});
 }
 
 int cmm_dot(cmm_op* op, const double* x, const double* y, int64_t n, double* result_host) {
@@ -1190,6 +1191,14 @@ static int solve_iteration(cmm_op* op, cmm_precon* pc, double* x, const SolveBuf
   const int64_t n = (int64_t)op->pt->ncomp * op->pt->npix;
   cudaStream_t st = op->ctx->stream;
   const bool ring = fcg.win > 1;
+  if (!flexible && !ring && !snap.buf) {
+    // plain PCG: the scalars are formed inside the vector kernels
+    CMM_TRY(apply_A_dev(op, v.p, v.q, v.cg_f32 ? nullptr : v.p1));
+    if (v.cg_f32) CMM_TRY(launch_dot_partial_cg(v.p, v.q, n, dst, v.p1, st));
+    CMM_TRY(launch_cg_step(dst, v.p1, x, v.r, v.p, v.q, n, v.p2, anorm, st));
+    CMM_TRY(precon_step(op, pc, v, dst, false));
+    return launch_cg_dir(dst, v.p2, v.p1, v.p, v.z, n, hist, st);
+  }
   CMM_TRY(apply_A_dev(op, v.p, v.q));
   CMM_TRY(launch_dot_partial_cg(v.p, v.q, n, dst, v.p1, st));
   CMM_TRY(launch_solver_alpha(dst, v.p1, anorm, st));
@@ -1343,7 +1352,7 @@ int cmm_solve(cmm_op* op, cmm_precon* pc, const double* b, double* x, const cmm_
   }
   const bool resume = opts->resume != 0;
   if (resume) {
-    h.rho = op->resume_rho;
+    h.rho = h.rho_new = op->resume_rho;
     h.iter = op->resume_iter;
     h.rel = op->resume_rel;
     h.status = CMM_ERR_NOT_CONVERGED;

@@ -223,15 +223,22 @@ inline TwLayout tw_layout(int R, int C) {
 
 // ---- launchers implemented in tod.cu
 int launch_map_to_gather(cmm_op* op, const double* m, bool clear_acc);
-int launch_acc_to_map(cmm_op* op, double* out);
+// The result map of an application and, with dot, the kRedBlocks partial sums of
+// dot^T map that its last kernel forms.
+struct ApplyOut {
+  double* map = nullptr;
+  const double* dot = nullptr;
+  double* partial = nullptr;
+};
+int launch_acc_to_map(cmm_op* op, double* out, const double* dot, double* partial);
 // Whether the last binning launch of an application writes the result itself, and whether
 // the FP64 accumulator takes part (else it needs no clearing).
 bool apply_direct(const cmm_op* op);
 bool apply_uses_acc(const cmm_op* op);
-// out: the result map, which the last chunk of a direct application writes (else unused)
-int launch_apply_chunk(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, double* out, int pass = -1);
+// out: written by the last chunk of a direct application (else unused)
+int launch_apply_chunk(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, const ApplyOut& out, int pass = -1);
 // out = P^T N^-1 P m, or P^T N^-1 tod where tod is given
-int launch_apply(cmm_op* op, const double* m, const void* tod, int tod_is_f64, double* out);
+int launch_apply(cmm_op* op, const double* m, const void* tod, int tod_is_f64, const ApplyOut& out);
 int launch_project(cmm_op* op, const double* m, void* tod, int tod_is_f64);
 int launch_hit_blocks(cmm_pointing* pt, const double* det_weight, const uint8_t* mask, double* blocks);
 int op_init_twiddles(cmm_op* op);
@@ -246,7 +253,7 @@ bool pair_path_fits(const cmm_op* op);
 bool pair_path_ok(const cmm_op* op);
 int pair_corr_slots_of(const cmm_op* op);   // bin slots of the correlated-noise tables
 bool pair_path_sizes(int log_nt, int* logR, int* logC);
-int launch_apply_chunk_pair(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, double* out, int pass);
+int launch_apply_chunk_pair(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, const ApplyOut& out, int pass);
 int launch_apply_chunk_pair64(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, int pass);
 int prepare_pair(cmm_op* op);
 int prepare_pair64(cmm_op* op);

@@ -339,7 +339,7 @@ __global__ void k_solver_beta(SolverDev* st, const double* __restrict__ p_rz, co
       return;
     }
     st->beta = cg_round(st, (p_flex ? fl : rz) / st->rho);
-    st->rho = rz;
+    st->rho = st->rho_new = rz;
   }
 }
 
@@ -352,6 +352,99 @@ __global__ void k_update_p(double* __restrict__ p, const double* __restrict__ z,
     p[i] = cg_round(st, z[i] + beta * p[i]);
 }
 
+// ------------------------------------------------------------------ the plain PCG step in two kernels
+// Every block forms the scalars itself from the partial sums (8 KB of L2; one warp a sum
+// and one thread for the divisions, since the FP64 pipe takes 16 cycles an instruction), so
+// no single-block kernel stands between the vector kernels.  With p^T q formed by the
+// application's last kernel an iteration is 10 kernels instead of 15: 20 circulant
+// iterations at 128 x 2^18 on 256 x 256 6.70 -> 6.1 ms; the two kernels take 7 us each at
+// 64 x 64, where the five and the dot product took 22.
+// What a kernel's blocks read, that kernel's block 0 does not write: rho is read by
+// k_cg_dir and written by k_cg_step, rho_new the other way round, and iter is read by
+// k_cg_dir and counted by k_cg_step.  `done` may be set while blocks of the same kernel
+// start: they then stop where they would have decided to stop.
+
+// alpha = rho / p^T q (or the breakdown), x += alpha p, r -= alpha q, partials of r^T r
+__global__ void __launch_bounds__(256) k_cg_step(SolverDev* st, const double* __restrict__ pq_part, double* __restrict__ x,
+                                                 double* __restrict__ r, const double* __restrict__ p,
+                                                 const double* __restrict__ q, long long n,
+                                                 double* __restrict__ rr_part, double* anorm_terms) {
+  if (st->done) return;
+  const double pq = partials_sum(pq_part, nullptr).x;
+  __shared__ double sh_alpha;   // NaN: breakdown
+  if (threadIdx.x == 0) {       // one thread: a division by every warp would cost more than the update
+    const double rho = st->rho_new;
+    const bool bad = !(pq > 0.0) || !isfinite(pq) || !isfinite(rho);
+    const double alpha = bad ? 0.0 : cg_round(st, rho / pq);
+    sh_alpha = bad ? nan("") : alpha;
+    if (blockIdx.x == 0) {
+      st->pq = pq;
+      st->rho = rho;
+      st->alpha = alpha;
+      if (bad) {
+        st->status = CMM_ERR_BREAKDOWN;
+        st->done = 1;
+      } else {
+        if (anorm_terms) anorm_terms[st->iter] = alpha * rho;
+        st->iter += 1;
+      }
+    }
+  }
+  __syncthreads();
+  const double alpha = sh_alpha;
+  if (isnan(alpha)) return;
+  double acc = 0.0;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    x[i] = cg_round(st, x[i] + alpha * p[i]);
+    const double ri = cg_round(st, r[i] - alpha * q[i]);
+    r[i] = ri;
+    acc = cg_acc(st, acc, ri * ri);
+  }
+  partial_store(acc, rr_part);
+}
+
+// After z = M r: the convergence check of the step just taken, beta = r^T z / rho and
+// p = z + beta p.  (The preconditioner has then run once more than a check between the two
+// would let it, on the last iteration only.)
+__global__ void __launch_bounds__(256) k_cg_dir(SolverDev* st, const double* __restrict__ rr_part,
+                                                const double* __restrict__ rz_part, double* __restrict__ p,
+                                                const double* __restrict__ z, long long n, double* hist) {
+  if (st->done) return;
+  const double2 sums = partials_sum(rr_part, rz_part);
+  __shared__ double sh_beta;
+  __shared__ int sh_status;   // -1: go on
+  if (threadIdx.x == 0) {
+    const double rr = sums.x, rz = sums.y;
+    const double rel = sqrt(rr / st->bnorm2);
+    const int iter = st->iter;
+    int status = -1;
+    if (!isfinite(rr)) status = CMM_ERR_BREAKDOWN;
+    else if (rel <= st->tol) status = CMM_OK;
+    else if (iter >= st->maxit) status = CMM_ERR_NOT_CONVERGED;
+    else if (!(rz > 0.0) || !isfinite(rz)) status = CMM_ERR_BREAKDOWN;
+    const double beta = cg_round(st, rz / st->rho);
+    sh_beta = beta;
+    sh_status = status;
+    if (blockIdx.x == 0) {
+      st->rr = rr;
+      if (hist) hist[iter] = rel;
+      if (isfinite(rr)) st->rel = rel;   // else the last finite residual stays
+      if (status >= 0) {
+        st->status = status;
+        st->done = 1;
+      } else {
+        st->beta = beta;
+        st->rho_new = rz;
+      }
+    }
+  }
+  __syncthreads();
+  if (sh_status >= 0) return;
+  const double beta = sh_beta;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    p[i] = cg_round(st, z[i] + beta * p[i]);
+}
+
 // Initialisation after r0, z0 are known: rho = r^T z (partial), bnorm2 set by host.
 __global__ void k_solver_init(SolverDev* st, const double* __restrict__ partial_rz,
                               const double* __restrict__ partial_rr, double* hist) {
@@ -359,7 +452,7 @@ __global__ void k_solver_init(SolverDev* st, const double* __restrict__ partial_
   __syncthreads();
   const double rr = block_sum_all(partial_rr, kRedBlocks);
   if (threadIdx.x == 0) {
-    st->rho = rz;
+    st->rho = st->rho_new = rz;
     st->iter = 0;
     const double rel = sqrt(rr / st->bnorm2);
     st->rel = isfinite(rel) ? rel : -1.0;   // -1: the starting residual is not finite
@@ -525,7 +618,7 @@ __global__ void k_solver_rho(SolverDev* st, const double* __restrict__ p_rz) {
       st->done = 1;
       return;
     }
-    st->rho = rz;
+    st->rho = st->rho_new = rz;
   }
 }
 
@@ -1155,6 +1248,26 @@ int launch_solver_beta(SolverDev* st, const double* p_rz, const double* p_flex, 
 
 int launch_update_p(double* p, const double* z, int64_t n, const SolverDev* st, cudaStream_t s) {
   k_update_p<<<grid_for(n), 256, 0, s>>>(p, z, n, st);
+  CMM_LAUNCH_CHECK();
+  return CMM_OK;
+}
+
+// Two blocks per SM while the partial sums that every block forms weigh, four for maps of
+// more than a million values.
+static int cg_blocks(int64_t n) { return n > (1 << 20) ? 608 : 304; }
+
+int launch_cg_step(SolverDev* st, const double* pq_part, double* x, double* r, const double* p, const double* q, int64_t n,
+                   double* rr_part, double* anorm, cudaStream_t s) {
+  const int g = (int)std::min<int64_t>((n + 255) / 256, cg_blocks(n));
+  k_cg_step<<<g, 256, 0, s>>>(st, pq_part, x, r, p, q, n, rr_part, anorm);
+  CMM_LAUNCH_CHECK();
+  return CMM_OK;
+}
+
+int launch_cg_dir(SolverDev* st, const double* rr_part, const double* rz_part, double* p, const double* z, int64_t n,
+                  double* hist, cudaStream_t s) {
+  const int g = (int)std::min<int64_t>((n + 255) / 256, cg_blocks(n));
+  k_cg_dir<<<g, 256, 0, s>>>(st, rr_part, rz_part, p, z, n, hist);
   CMM_LAUNCH_CHECK();
   return CMM_OK;
 }

@@ -13,6 +13,7 @@ constexpr int kMaxWin = 8;   // directions kept by truncated flexible CG, FCG(m)
 struct SolverDev {
   double rho, pq, alpha, beta, rr, rel, bnorm2, tol;
   int iter, maxit, done, status;
+  double rho_new; // r^T z for the next step (k_cg_step takes it over into rho)
   int f32;        // FP32 CG vectors and scalars
   int win;        // FCG(m): m > 1 directions kept (ring slot j mod m); <= 1: PCG / Polak-Ribiere
   double pq_ring[kMaxWin];   // p_j^T A p_j of the kept directions
@@ -68,6 +69,47 @@ __device__ __forceinline__ void mode_mul3(const H* __restrict__ o, const H (&xr)
   yi[2] = (h02r * xi[0] - h02i * xr[0]) + (h12r * xi[1] - h12i * xr[1]) + o[2] * xi[2];
 }
 
+// Fixed-order sum over a block of any whole number of warps (at most 32), in thread 0.
+__device__ __forceinline__ double block_sum_warps(double v) {
+  __shared__ double sh3[32];
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) sh3[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double r = 0.0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < (int)blockDim.x / 32; ++w) r += sh3[w];
+  return r;
+}
+
+// Sums of the kRedBlocks partials a (and b, if given), in every thread of a block that asks
+// and the same in every block.  One warp a sum: 37 instructions of the FP64 pipe, which a
+// sum by the whole block would give ten times as many.
+__device__ __forceinline__ double2 partials_sum(const double* __restrict__ a, const double* __restrict__ b) {
+  __shared__ double sh4[2];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const double* p = w == 0 ? a : b;
+  if (w < 2 && p) {
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 2
+    for (int i = lane; i < kRedBlocks; i += 128)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[j] += p[i + 32 * j];
+    double s = (v[0] + v[1]) + (v[2] + v[3]);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) sh4[w] = s;
+  }
+  __syncthreads();
+  return double2{sh4[0], b ? sh4[1] : 0.0};
+}
+
+// A block's sum into its partial; block 0 clears the partials past the grid.
+__device__ __forceinline__ void partial_store(double v, double* partial) {
+  const double s = block_sum_warps(v);
+  if (threadIdx.x == 0) partial[blockIdx.x] = s;
+  if (blockIdx.x == 0)
+    for (int b = gridDim.x + threadIdx.x; b < kRedBlocks; b += blockDim.x) partial[b] = 0.0;
+}
+
 int launch_block_apply_dot(int ncomp, int64_t npix, const double* blk, const double* x, double* y,
                            const double* w, double* partial, const int* done, cudaStream_t s);
 // y = d .* x and z = (first ? 0 : z) + d .* x on every Stokes component (d [npix])
@@ -91,6 +133,10 @@ int launch_residual(double* r, const double* b, const double* q, int64_t n, cons
 int launch_solver_rho(SolverDev* st, const double* p_rz, cudaStream_t s);
 int launch_snapshot(const double* x, const double* r, int64_t n, const SolverDev* st, int every, int max,
                     double* snaps, cudaStream_t s);
+int launch_cg_step(SolverDev* st, const double* pq_part, double* x, double* r, const double* p, const double* q, int64_t n,
+                   double* rr_part, double* anorm, cudaStream_t s);
+int launch_cg_dir(SolverDev* st, const double* rr_part, const double* rz_part, double* p, const double* z, int64_t n,
+                  double* hist, cudaStream_t s);
 int launch_solver_check(SolverDev* st, const double* partial, double* hist, cudaStream_t s);
 int launch_solver_beta(SolverDev* st, const double* p_rz, const double* p_flex, cudaStream_t s);
 int launch_update_p(double* p, const double* z, int64_t n, const SolverDev* st, cudaStream_t s);

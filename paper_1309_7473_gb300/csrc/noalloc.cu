@@ -87,7 +87,7 @@ int cmm_apply_A_noalloc(cmm_op* op, const double* m_in, double* m_out) {
   // The array keeps whatever the previous call left: the FP32 partial map must
   // start at zero (the FP64 accumulator is cleared with the gather copy where it is used).
   CMM_CUDA(cudaMemsetAsync(v.acc32, 0, sizeof(float) * op->acc_stride * (npix + 1), op->ctx->stream));
-  return launch_apply(&v, m_in, nullptr, 0, m_out);
+  return launch_apply(&v, m_in, nullptr, 0, ApplyOut{m_out});
 }
 
 }  // extern "C"

@@ -20,6 +20,7 @@
 
 #include "common.cuh"
 #include "fft.cuh"
+#include "map_kernels.cuh"
 #include "tod_common.cuh"
 #include "tod_fast.cuh"
 
@@ -201,16 +202,24 @@ __global__ void k_map_to_gather(const double* __restrict__ m, const uint8_t* __r
   }
 }
 
+// dot (may be nullptr): the partial sums of dot^T out over the grid
 template <int NC>
 __global__ void k_acc_to_map(const double* __restrict__ acc, const uint8_t* __restrict__ mask,
-                             double* __restrict__ out, int acc_stride, long long npix, const int* done) {
+                             double* __restrict__ out, int acc_stride, long long npix, const double* __restrict__ dot,
+                             double* __restrict__ partial, const int* done) {
   if (done && *done) return;
+  double sum = 0.0;
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < npix;
        p += (long long)gridDim.x * blockDim.x) {
     const bool ok = mask[p] != 0;
 #pragma unroll
-    for (int c = 0; c < NC; ++c) out[c * npix + p] = ok ? acc[p * acc_stride + c] : 0.0;
+    for (int c = 0; c < NC; ++c) {
+      const double v = ok ? acc[p * acc_stride + c] : 0.0;
+      out[c * npix + p] = v;
+      if (dot) sum += dot[c * npix + p] * v;
+    }
   }
+  if (dot) partial_store(sum, partial);
 }
 
 // tod[d][t] = (P m)_{d,t}: pointing + gather only (used to synthesise noise-free data).
@@ -414,13 +423,15 @@ int launch_map_to_gather(cmm_op* op, const double* m, bool clear_acc) {
   return f64 ? map_to_gather_t<double, 3>(op, m, clear_acc) : map_to_gather_t<float, 3>(op, m, clear_acc);
 }
 
-int launch_acc_to_map(cmm_op* op, double* out) {
+int launch_acc_to_map(cmm_op* op, double* out, const double* dot, double* partial) {
   const long long npix = op->pt->npix;
-  const int blocks = (int)std::min<long long>((npix + 255) / 256, 4096);
+  const int blocks = (int)std::min<long long>((npix + 255) / 256, dot ? kRedBlocks : 4096);
   if (op->pt->ncomp == 1)
-    k_acc_to_map<1><<<blocks, 256, 0, op->ctx->stream>>>(op->acc, op->pt->mask, out, op->acc_stride, npix, op->done);
+    k_acc_to_map<1><<<blocks, 256, 0, op->ctx->stream>>>(op->acc, op->pt->mask, out, op->acc_stride, npix, dot, partial,
+                                                         op->done);
   else
-    k_acc_to_map<3><<<blocks, 256, 0, op->ctx->stream>>>(op->acc, op->pt->mask, out, op->acc_stride, npix, op->done);
+    k_acc_to_map<3><<<blocks, 256, 0, op->ctx->stream>>>(op->acc, op->pt->mask, out, op->acc_stride, npix, dot, partial,
+                                                         op->done);
   CMM_LAUNCH_CHECK();
   return CMM_OK;
 }
@@ -488,7 +499,7 @@ static int apply_chunk_nc(cmm_op* op, int d0, int nd, const void* tod, int pass)
   }
 }
 
-int launch_apply_chunk(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, double* out, int pass) {
+int launch_apply_chunk(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, const ApplyOut& out, int pass) {
   const int nc = op->pt->ncomp;
   if (pair_path_ok(op)) return launch_apply_chunk_pair(op, d0, nd, tod, tod_is_f64, out, pass);
   if (fast_path_ok(op)) {
@@ -515,7 +526,7 @@ bool apply_uses_acc(const cmm_op* op) {
   return !apply_direct(op) || op->chunk < op->pt->n_det || op->pt->n_det > op->acc32_maps * kFlushDets;
 }
 
-int launch_apply(cmm_op* op, const double* m, const void* tod, int tod_is_f64, double* out) {
+int launch_apply(cmm_op* op, const double* m, const void* tod, int tod_is_f64, const ApplyOut& out) {
   const bool acc = apply_uses_acc(op);
   if (!tod) CMM_TRY(launch_map_to_gather(op, m, acc));
   else if (acc)
@@ -524,7 +535,7 @@ int launch_apply(cmm_op* op, const double* m, const void* tod, int tod_is_f64, d
     const int nd = std::min(op->chunk, op->pt->n_det - d0);
     CMM_TRY(launch_apply_chunk(op, d0, nd, tod, tod_is_f64, out));
   }
-  return apply_direct(op) ? CMM_OK : launch_acc_to_map(op, out);
+  return apply_direct(op) ? CMM_OK : launch_acc_to_map(op, out.map, out.dot, out.partial);
 }
 
 int launch_generic_fwd_from_tod(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64) {

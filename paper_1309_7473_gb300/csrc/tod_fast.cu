@@ -30,6 +30,7 @@
 
 #include "common.cuh"
 #include "fft_reg.cuh"
+#include "map_kernels.cuh"
 #include "tod_common.cuh"
 #include "tod_fast.cuh"
 
@@ -714,8 +715,9 @@ __global__ void k_fast_flush_maps(float* __restrict__ acc32, int maps, long long
 template <int NC>
 __global__ void k_flush_to_map(float* __restrict__ acc32, int maps, long long map_elems, const double* __restrict__ acc,
                                const uint8_t* __restrict__ mask, double* __restrict__ out, long long npix,
-                               const int* done) {
+                               const double* __restrict__ dot, double* __restrict__ partial, const int* done) {
   if (done && *done) return;
+  double sum = 0.0;   // of dot^T out
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < npix;
        p += (long long)gridDim.x * blockDim.x) {
     const bool ok = mask[p] != 0;
@@ -729,7 +731,9 @@ __global__ void k_flush_to_map(float* __restrict__ acc32, int maps, long long ma
           *q = 0.0f;
         }
       }
-      out[p] = ok ? s : 0.0;
+      s = ok ? s : 0.0;
+      out[p] = s;
+      if (dot) sum += dot[p] * s;
     } else {
       double s0 = 0.0, s1 = 0.0, s2 = 0.0;
       if (acc) {
@@ -747,19 +751,28 @@ __global__ void k_flush_to_map(float* __restrict__ acc32, int maps, long long ma
           *q = make_float4(0.f, 0.f, 0.f, 0.f);
         }
       }
-      out[p] = ok ? s0 : 0.0;
-      out[npix + p] = ok ? s1 : 0.0;
-      out[2 * npix + p] = ok ? s2 : 0.0;
+      s0 = ok ? s0 : 0.0;
+      s1 = ok ? s1 : 0.0;
+      s2 = ok ? s2 : 0.0;
+      out[p] = s0;
+      out[npix + p] = s1;
+      out[2 * npix + p] = s2;
+      if (dot) sum += dot[p] * s0 + dot[npix + p] * s1 + dot[2 * npix + p] * s2;
     }
   }
+  if (dot) partial_store(sum, partial);
 }
 
-int launch_flush_to_map(const TodArgs& a, int nc, int maps, bool add_acc, const uint8_t* mask, double* out,
+int launch_flush_to_map(const TodArgs& a, int nc, int maps, bool add_acc, const uint8_t* mask, const ApplyOut& out,
                         cudaStream_t st) {
-  const int blocks = (int)std::min<long long>((a.npix + 255) / 256, 4096);
+  const int blocks = (int)std::min<long long>((a.npix + 255) / 256, out.dot ? kRedBlocks : 4096);
   const double* acc = add_acc ? a.acc : nullptr;
-  if (nc == 1) k_flush_to_map<1><<<blocks, 256, 0, st>>>(a.acc32, maps, a.acc32_map, acc, mask, out, a.npix, a.done);
-  else k_flush_to_map<3><<<blocks, 256, 0, st>>>(a.acc32, maps, a.acc32_map, acc, mask, out, a.npix, a.done);
+  if (nc == 1)
+    k_flush_to_map<1><<<blocks, 256, 0, st>>>(a.acc32, maps, a.acc32_map, acc, mask, out.map, a.npix, out.dot, out.partial,
+                                              a.done);
+  else
+    k_flush_to_map<3><<<blocks, 256, 0, st>>>(a.acc32, maps, a.acc32_map, acc, mask, out.map, a.npix, out.dot, out.partial,
+                                              a.done);
   CMM_LAUNCH_CHECK();
   return CMM_OK;
 }

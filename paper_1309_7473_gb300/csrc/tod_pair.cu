@@ -24,7 +24,7 @@ int pair_corr_slots_of(const cmm_op* op) { return pair_corr_slots(op->pR, op->pC
 
 bool pair_path_ok(const cmm_op* op) { return op->pair && pair_path_fits(op); }
 
-int launch_flush_to_map(const TodArgs& a, int nc, int maps, bool add_acc, const uint8_t* mask, double* out,
+int launch_flush_to_map(const TodArgs& a, int nc, int maps, bool add_acc, const uint8_t* mask, const ApplyOut& out,
                         cudaStream_t st);
 int launch_flush_maps(const TodArgs& a, int nc, int maps, cudaStream_t st);
 
@@ -43,7 +43,7 @@ static int run_corr(const TodArgs& a, int nd, cudaStream_t st) {
 static_assert(kMaxCorrModes == 4, "k_pair_corr instances");
 
 template <typename S>
-static int apply_pair_s(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, double* out, int pass) {
+static int apply_pair_s(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, const ApplyOut& out, int pass) {
   TodArgs a = pair_args(op, d0);
   a.tod = tod;
   cudaStream_t st = op->ctx->stream;
@@ -90,7 +90,7 @@ static int apply_pair_s(cmm_op* op, int d0, int nd, const void* tod, int tod_is_
 }
 
 // tod: stored data [n_det][n_t] in place of P m, or nullptr.
-int launch_apply_chunk_pair(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, double* out, int pass) {
+int launch_apply_chunk_pair(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, const ApplyOut& out, int pass) {
   if (op->prec == CMM_PREC_F64) return launch_apply_chunk_pair64(op, d0, nd, tod, tod_is_f64, pass);
   if (op->prec == CMM_PREC_BF16) return apply_pair_s<__nv_bfloat162>(op, d0, nd, tod, tod_is_f64, out, pass);
   return apply_pair_s<float2>(op, d0, nd, tod, tod_is_f64, out, pass);
