@@ -690,7 +690,7 @@ SETUP_LAUNCHES = 4
 
 # sources of the three A-application kernels of the two-detector path: the traffic
 # record holds for them only
-TRAFFIC_SOURCES = ("tod_pair.cu", "tod_fast.cuh", "fft_reg.cuh", "fft.cuh", "tod_common.cuh", "common.cuh")
+TRAFFIC_SOURCES = ("tod_pair.cuh", "tod_fast.cuh", "fft_reg.cuh", "fft.cuh", "tod_common.cuh", "common.cuh")
 
 
 def kernel_sources_digest():
