@@ -87,6 +87,20 @@ __device__ __forceinline__ Cx2<T> cx_scale(T c, const Cx2<T>& a) {
   const V2<T> cc{c, c};
   return Cx2<T>{pmul(cc, a.re), pmul(cc, a.im)};
 }
+// a (c + i s).  In FP32 with what the rounded constants lack, added before the products
+// are rounded: every butterfly uses the same constants, so their errors do not average out
+// over a line as those of the stage twiddles do.
+template <typename T>
+__device__ __forceinline__ Cx2<T> cx_mul_const(const Cx2<T>& a, double c, double s) {
+  if constexpr (sizeof(T) == 8) {
+    return cx_mul<T>(a, c, s);
+  } else {
+    const T ch = (T)c, sh = (T)s, cl = (T)(c - (double)ch), sl = (T)(s - (double)sh);
+    const V2<T> cc{ch, ch}, ss{sh, sh}, ns{-sh, -sh}, dc{cl, cl}, ds{sl, sl}, dn{-sl, -sl};
+    return Cx2<T>{pfma(a.im, ns, pfma(a.re, cc, pfma(a.im, dn, pmul(a.re, dc)))),
+                  pfma(a.re, ss, pfma(a.im, cc, pfma(a.re, ds, pmul(a.im, dc))))};
+  }
+}
 // x_q <- sum_j x_j exp(SIGN 2 pi i j q / N): direct forms for 2 to 5, N = A B else
 // (A-point transforms, the constants w_N^(b c), B-point transforms)
 template <typename T, int N, int SIGN>
@@ -129,7 +143,7 @@ __device__ __forceinline__ void cx_dft_n(Cx2<T>* x) {
           const Cx2<T> v = y[b][c];
           y[b][c] = SIGN > 0 ? Cx2<T>{V2<T>{-v.im.x, -v.im.y}, v.re} : Cx2<T>{v.im, V2<T>{-v.re.x, -v.re.y}};
         } else {
-          y[b][c] = cx_mul<T>(y[b][c], (T)wr, (T)wi);
+          y[b][c] = cx_mul_const<T>(y[b][c], wr, wi);
         }
       });
     });
