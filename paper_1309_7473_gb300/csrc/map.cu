@@ -361,15 +361,22 @@ __global__ void k_update_p(double* __restrict__ p, const double* __restrict__ z,
 // 64 x 64, where the five and the dot product took 22.
 // What a kernel's blocks read, that kernel's block 0 does not write: rho is read by
 // k_cg_dir and written by k_cg_step, rho_new the other way round, and iter is read by
-// k_cg_dir and counted by k_cg_step.  `done` may be set while blocks of the same kernel
-// start: they then stop where they would have decided to stop.
+// k_cg_dir and counted by k_cg_step.  `done` is the exception: block 0 may set it while
+// other blocks of the same kernel start.  Each block therefore reads it once, for all of
+// its threads (cg_done), and stays or leaves as a whole; one that leaves on the new value
+// does what its own decision would have been, since every block forms the same scalars.
+
+// One thread's read of st->done, the same answer in every thread of the block.
+__device__ __forceinline__ bool cg_done(const SolverDev* st) {
+  return __syncthreads_or(threadIdx.x == 0 && *(const volatile int*)&st->done) != 0;
+}
 
 // alpha = rho / p^T q (or the breakdown), x += alpha p, r -= alpha q, partials of r^T r
 __global__ void __launch_bounds__(256) k_cg_step(SolverDev* st, const double* __restrict__ pq_part, double* __restrict__ x,
                                                  double* __restrict__ r, const double* __restrict__ p,
                                                  const double* __restrict__ q, long long n,
                                                  double* __restrict__ rr_part, double* anorm_terms) {
-  if (st->done) return;
+  if (cg_done(st)) return;
   const double pq = partials_sum(pq_part, nullptr).x;
   __shared__ double sh_alpha;   // NaN: breakdown
   if (threadIdx.x == 0) {       // one thread: a division by every warp would cost more than the update
@@ -409,7 +416,7 @@ __global__ void __launch_bounds__(256) k_cg_step(SolverDev* st, const double* __
 __global__ void __launch_bounds__(256) k_cg_dir(SolverDev* st, const double* __restrict__ rr_part,
                                                 const double* __restrict__ rz_part, double* __restrict__ p,
                                                 const double* __restrict__ z, long long n, double* hist) {
-  if (st->done) return;
+  if (cg_done(st)) return;
   const double2 sums = partials_sum(rr_part, rz_part);
   __shared__ double sh_beta;
   __shared__ int sh_status;   // -1: go on
