@@ -219,14 +219,18 @@ int cmm_op_destroy(cmm_op* op);
  * BF16 operators of non-periodic maps (else CMM_ERR_UNSUPPORTED). */
 int cmm_op_set_pixel_cache(cmm_op* op, int32_t enable);
 /* Two-detector FFT packing of A and of the right-hand side (enable != 0, the default):
- * for 2^13 <= n_samp <= 2^20, the
- * noise filter of Sec. Test setup is applied to two detectors at once as one
- * complex sequence z = s_1 + i s_2 of n_samp points, so that every complex element
+ * for 2^13 <= n_samp <= 2^20, the noise filter of Sec. Test setup is applied to two
+ * detectors at once as one complex sequence z = s_1 + i s_2 of n_samp points, so that every complex element
  * is one time sample of both and the pointing tables are read once for the two;
  * each bin pair (k, n - k) is filtered as Y(k) = a Z(k) + b conj Z(n - k) with
- * a, b = (w_1 +- w_2) / 2.  enable == 0 selects the one-detector packing (even
- * and odd samples as one complex sequence of n_samp / 2 points), which also serves
- * operators above the FP32 hit limit.
+ * a, b = (w_1 +- w_2) / 2.  The rounding of a sequence is that of its larger member, so
+ * weights and stored data travel in powers of two per detector that bring the two to the
+ * same size, for stored data from their measured level: a loud detector (a glitch, a
+ * drift, garbage under a weight of zero, which is not looked at) leaves its partner's
+ * accuracy as it is, and NaN or Inf stay with their detector unless the noise is
+ * correlated.  enable == 0 selects the one-detector packing (even and odd samples as one
+ * complex sequence of n_samp / 2 points), which also serves operators above the FP32 hit
+ * limit.
  * Results agree to the rounding of the spectrum storage (FP64, FP32 or BF16) either way;
  * waits for the operator's stream. */
 int cmm_op_set_pair_packing(cmm_op* op, int32_t enable);

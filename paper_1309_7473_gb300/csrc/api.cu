@@ -305,6 +305,7 @@ static void free_noise(cmm_noise* nz) {
   dfree(nz->coef32);
   dfree(nz->diag);
   dfree(nz->white);
+  dfree(nz->pair64);
   dfree(nz->corr_V);
   dfree(nz->corr_par);
   dfree(nz->wtab64);
@@ -320,6 +321,50 @@ static void noise_release(cmm_noise* nz) {
 
 int cmm_noise_destroy(cmm_noise* nz) {
   if (nz) noise_release(nz);
+  return CMM_OK;
+}
+
+// The power of two nearest v > 0 (0 else), within 2^+-60 so that products and quotients of
+// two of them are exact in FP32.
+static float near_pow2(double v) {
+  if (!(v > 0)) return 0.0f;
+  return (float)std::exp2(std::min(60.0, std::max(-60.0, std::rint(std::log2(v)))));
+}
+
+// The units of the two-detector path from the root-mean-square weight of every detector
+// (the law's mean is within a factor of two of it at the usual slopes).  Two detectors
+// share one complex sequence, so the rounding of the larger reaches the smaller: weights
+// are divided by u before the filter and the filtered data multiplied by it after, and
+// stored data, whose noise has variance 1 / w, by the guess before the transform.
+static int noise_units(cmm_noise* nz, const std::vector<double>& w) {
+  const size_t n = nz->n_det;
+  const size_t at32 = sizeof(double4_32a) * 2 * n, at_unit = at32 + sizeof(float4) * 2 * n;
+  const size_t at_guess = at_unit + sizeof(float) * 2 * n, bytes = at_guess + sizeof(float) * n;
+  std::vector<double4_32a> buf(bytes / sizeof(double4_32a) + 1);   // for its alignment
+  unsigned char* host = reinterpret_cast<unsigned char*>(buf.data());
+  double4_32a* c64 = buf.data();
+  float4* c32 = reinterpret_cast<float4*>(host + at32);
+  float* unit = reinterpret_cast<float*>(host + at_unit);
+  float* guess = reinterpret_cast<float*>(host + at_guess);
+  for (size_t d = 0; d < n; ++d) {
+    unit[d] = 1.0f;
+    unit[n + d] = near_pow2(w[d]);
+    guess[d] = near_pow2(std::sqrt(w[d]));
+    for (size_t q = d; q < 2 * n; q += n) {
+      const float iu = unit[q] > 0 ? 1.0f / unit[q] : 0.0f;
+      const double4_32a c = nz->coef_host[d];
+      c64[q] = double4_32a{nz->wtab64 ? (double)iu : c.x * iu, c.y, c.z, c.w};
+      c32[q] = float4{nz->wtab64 ? iu : (float)c.x * iu, (float)c.y, (float)c.z, (float)c.w};
+    }
+  }
+  if (!nz->pair64) {
+    CMM_TRY(dalloc(&nz->pair64, bytes));
+    unsigned char* dev = reinterpret_cast<unsigned char*>(nz->pair64);
+    nz->pair32 = reinterpret_cast<float4*>(dev + at32);
+    nz->unit = reinterpret_cast<float*>(dev + at_unit);
+    nz->tod_guess = reinterpret_cast<float*>(dev + at_guess);
+  }
+  CMM_CUDA(cudaMemcpy(nz->pair64, host, bytes, cudaMemcpyHostToDevice));
   return CMM_OK;
 }
 
@@ -368,7 +413,8 @@ int cmm_noise_create(cmm_ctx* ctx, int32_t n_det, int64_t n_samp, double f_samp,
     nz->diag_host.resize(n_det);
     CMM_CUDA(cudaMemcpyAsync(nz->diag_host.data(), nz->diag, sizeof(double) * n_det, cudaMemcpyDeviceToHost, st));
     CMM_CUDA(cudaStreamSynchronize(st));
-    return CMM_OK;
+    nz->coef_host = c64;
+    return noise_units(nz, nz->diag_host);
   };
   s = run();
   if (s != CMM_OK) {
@@ -397,6 +443,7 @@ static void free_op(cmm_op* op) {
   dfree(op->tw_pair);
   dfree(op->rot64);
   dfree(op->lg2);
+  dfree(op->tod_norm);
   dfree(op->tmp_a);
   dfree(op->tmp_b);
   dfree(op->pix);
@@ -518,13 +565,13 @@ int cmm_noise_set_table(cmm_noise* nz, const double* w_host) {
   nz->wtab64 = nullptr;
   nz->wtab32 = nullptr;
   nz->corr_version++;   // correlated-noise tables depend on the weights
-  std::vector<double> diag(n_det);
+  std::vector<double> diag(n_det), rms(n_det);
   if (!w_host) {
     k_noise_diag<<<n_det, 256, 0, st>>>(nz->coef64, nz->n_t, nz->diag);
     CMM_LAUNCH_CHECK();
     CMM_CUDA(cudaMemcpyAsync(nz->diag_host.data(), nz->diag, sizeof(double) * n_det, cudaMemcpyDeviceToHost, st));
     CMM_CUDA(cudaStreamSynchronize(st));
-    return CMM_OK;
+    return noise_units(nz, nz->diag_host);
   }
   std::vector<float> w32((size_t)n_det * K);
   for (int d = 0; d < n_det; ++d) {
@@ -532,7 +579,14 @@ int cmm_noise_set_table(cmm_noise* nz, const double* w_host) {
     double inner = 0.0;   // R3: mean of w over the full two-sided grid
     for (int64_t k = 1; k < K - 1; ++k) inner += w[k];
     diag[d] = (w[0] + 2.0 * inner + w[K - 1]) / (double)nz->n_t;
-    for (int64_t k = 0; k < K; ++k) w32[(size_t)d * K + k] = (float)w[k];
+    const double top = *std::max_element(w, w + K);
+    double sq = 0.0;   // of w / top, which cannot overflow
+    for (int64_t k = 0; k < K; ++k) {
+      const double v = top > 0 ? w[k] / top : 0.0;
+      sq += v * v;
+      w32[(size_t)d * K + k] = (float)w[k];
+    }
+    rms[d] = top * std::sqrt(sq / (double)K);
   }
   CMM_TRY(dalloc(&nz->wtab64, sizeof(double) * (size_t)n_det * K));
   CMM_TRY(dalloc(&nz->wtab32, sizeof(float) * (size_t)n_det * K));
@@ -540,7 +594,7 @@ int cmm_noise_set_table(cmm_noise* nz, const double* w_host) {
   CMM_CUDA(cudaMemcpy(nz->wtab32, w32.data(), sizeof(float) * (size_t)n_det * K, cudaMemcpyHostToDevice));
   CMM_CUDA(cudaMemcpy(nz->diag, diag.data(), sizeof(double) * n_det, cudaMemcpyHostToDevice));
   nz->diag_host = diag;
-  return CMM_OK;
+  return noise_units(nz, rms);
 }
 
 int cmm_noise_set_correlated(cmm_noise* nz, int32_t r, const double* modes, const double* amp, const double* fknee,

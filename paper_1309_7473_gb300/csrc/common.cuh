@@ -156,6 +156,15 @@ struct cmm_noise {
   double* diag = nullptr;      // [n_det] diag(N^-1)
   double* white = nullptr;     // [n_det] 1 / sigma^2, the white level of the law
   std::vector<double> diag_host;
+  // two-detector path (noise_units, api.cu), [2][n_det] each, for A and for the right-hand
+  // side: the unit u of the weights (a power of two; 0 without weight) and the coefficients
+  // with 1 / sigma^2 in that unit (with a table: 1 / u, its factor)
+  // (one allocation, at pair64)
+  double4_32a* pair64 = nullptr;
+  float4* pair32 = nullptr;
+  float* unit = nullptr;
+  float* tod_guess = nullptr;   // [n_det] factor that makes data of this noise of order one
+  std::vector<double4_32a> coef_host;
   // noise correlated between detectors: N(f) = D(f) + V E(f) V^T (r modes, 0 = none)
   int corr_r = 0;
   int corr_version = 0;        // bumped by every cmm_noise_set_correlated
@@ -185,6 +194,13 @@ struct cmm_op {
   void* tw_pair = nullptr;     // their twiddle tables (the op's compute type)
   double2* rot64 = nullptr;    // FP64 two-detector path: [n_t] (cos 2phi, sin 2phi)
   double* lg2 = nullptr;       // the same: [n_t / 2 + 1] log2 of the frequency index, 64 powers 2^(j / 64)
+  // two-detector path from stored data: [n_det] sums of squares (zero between calls), the
+  // factors on the data and on the filtered data, and the pairs to transform again (one
+  // allocation, at tod_norm)
+  double* tod_norm = nullptr;
+  float* tod_f = nullptr;
+  float* tod_h = nullptr;
+  int* tod_list = nullptr;     // [1 + pairs]: their number, then the pairs
   int corr_version = 0;        // noise correlation version the tables below were built for
   float* corr_minv = nullptr;  // per-bin M^-1, [r][r] each, in the slot order of the path in use
   float2* corr_s = nullptr;    // cross-detector solution per bin slot ([slots][r], two-detector path [r][slots])

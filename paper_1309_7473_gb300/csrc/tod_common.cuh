@@ -101,6 +101,11 @@ struct TodArgs {
   const float* corrV;   // [n_det][corr_r]
   const float* corr_minv;   // [N + 1][r][r] slot order
   float2* corr_s;       // [N][r]
+  // two-detector path, per detector: factor on the data (nullptr: 1) and on the filtered data
+  const float* tod_f;
+  const float* tod_h;
+  double* tod_norm;     // sums of squares of stored data, times tod_f^2
+  const int* tod_list;  // pairs to transform again
   int d0;
   const int* done;
 };
@@ -198,6 +203,10 @@ static inline TodArgs make_args(const cmm_op* op, int d0) {
   a.corrV = op->nz->corr_V;
   a.corr_minv = op->corr_minv;
   a.corr_s = op->corr_s;
+  a.tod_f = nullptr;
+  a.tod_h = op->nz->unit;
+  a.tod_norm = op->tod_norm;
+  a.tod_list = op->tod_list;
   a.d0 = d0;
   a.done = op->done;
   return a;

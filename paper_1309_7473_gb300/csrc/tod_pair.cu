@@ -1,5 +1,6 @@
 // Two-detector path of the FP32 and BF16 operators: sizes, tables and launches of the
 // kernels of tod_pair.cuh.
+#include "map_kernels.cuh"
 #include "tod_pair.cuh"
 
 namespace cmm {
@@ -28,6 +29,92 @@ int launch_flush_to_map(const TodArgs& a, int nc, int maps, bool add_acc, const 
                         cudaStream_t st);
 int launch_flush_maps(const TodArgs& a, int nc, int maps, cudaStream_t st);
 
+// ------------------------------------------------------------------ factors of stored data
+// One block after the first forward pass: from every detector's sum of squares (cleared for
+// the next call) its factors f and h = u / f, and the list of pairs to transform again.
+//
+// level = mean square of f s.  A pair whose rms differ by less than kTodBalance keeps the
+// guesses: its quieter detector then carries at most about kTodBalance times its own
+// rounding (FP32 2.5e-7, alone 3e-7).  Else both take the power of two nearest 1 / rms.
+// Without weight: f = h = 0, and for an all-zero detector h = 0, as their filtered data are
+// exactly zero.  Not finite: NaN for that detector alone, f = 0 keeps it out of its
+// partner's sequence.  With correlated noise a detector's filtered data also hold the common
+// modes, whose size is that of all detectors' data: no level is then taken below their
+// weighted mean square.
+constexpr double kTodBalance = 4.0;
+constexpr int kGainThreads = 1024;
+
+__global__ void __launch_bounds__(kGainThreads) k_tod_gains(double* norm, const float* __restrict__ guess,
+                                                            const float* __restrict__ unit, float* __restrict__ f,
+                                                            float* __restrict__ h, int* __restrict__ list, int d0, int nd,
+                                                            double per, bool corr, const int* done) {
+  if (done && *done) return;
+  __shared__ int count;
+  __shared__ double common;
+  if (threadIdx.x == 0) count = 0;
+  if (corr) {
+    double su = 0.0, sr = 0.0;
+    for (int d = d0 + threadIdx.x; d < d0 + nd; d += kGainThreads) {
+      const double f0 = (double)guess[d], ms = norm[d] * per;
+      if (f0 > 0.0 && isfinite(ms)) {
+        su += (double)unit[d];
+        sr += (double)unit[d] * (ms / (f0 * f0));
+      }
+    }
+    su = block_sum_warps(su);
+    __syncthreads();
+    sr = block_sum_warps(sr);
+    if (threadIdx.x == 0) common = su > 0.0 ? sr / su : 0.0;
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; 2 * q < nd; q += kGainThreads) {
+    double level[2] = {0.0, 0.0};
+    bool again = false;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int d = d0 + 2 * q + j;
+      if (2 * q + j >= nd) break;
+      const double ms = norm[d] * per;
+      const float f0 = guess[d];
+      norm[d] = 0.0;
+      f[d] = f0;
+      if (f0 == 0.0f) {
+        h[d] = 0.0f;
+      } else if (!isfinite(ms)) {
+        f[d] = 0.0f;
+        h[d] = NAN;
+        again = true;
+      } else {
+        level[j] = corr ? fmax(ms, common * ((double)f0 * f0)) : ms;
+        h[d] = level[j] > 0.0 ? unit[d] / f0 : 0.0f;
+      }
+    }
+    if (level[0] > 0.0 && level[1] > 0.0 &&
+        fmax(level[0], level[1]) > kTodBalance * kTodBalance * fmin(level[0], level[1])) {
+      again = true;
+      for (int j = 0; j < 2; ++j) {
+        const int d = d0 + 2 * q + j;
+        // the guess over sqrt(level), within 2^+-100, and u / f within FP32
+        const int eu = ilogbf(unit[d]);
+        const int ef = (int)fmin(100.0, fmax(-100.0, ilogbf(guess[d]) - rint(0.5 * log2(level[j]))));
+        f[d] = scalbnf(1.0f, min(max(ef, eu - 126), eu + 126));
+        h[d] = unit[d] / f[d];
+      }
+    }
+    if (again) list[1 + atomicAdd(&count, 1)] = q;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) list[0] = count;
+}
+
+int launch_tod_gains(const cmm_op* op, const TodArgs& a, int nd, cudaStream_t st) {
+  k_tod_gains<<<1, kGainThreads, 0, st>>>(op->tod_norm, op->nz->tod_guess, op->nz->unit + op->pt->n_det, op->tod_f,
+                                          op->tod_h, op->tod_list, a.d0, nd, 1.0 / (double)op->pt->n_t, a.corr_r > 0,
+                                          a.done);
+  CMM_LAUNCH_CHECK();
+  return CMM_OK;
+}
+
 template <typename S>
 static int run_corr(const TodArgs& a, int nd, cudaStream_t st) {
   const int g = (pair_corr_slots(a.R, a.C) + kCorrThreads - 1) / kCorrThreads;
@@ -45,12 +132,12 @@ static_assert(kMaxCorrModes == 4, "k_pair_corr instances");
 template <typename S>
 static int apply_pair_s(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, const ApplyOut& out, int pass) {
   TodArgs a = pair_args(op, d0);
-  a.tod = tod;
+  if (tod) stored_gains(op, a);
   cudaStream_t st = op->ctx->stream;
   const int nc = op->pt->ncomp;
   if (pass < 0 || pass == 0) {
     TraceRange tr("A: P m + column FFTs (two detectors per sequence)");
-    if (tod) CMM_TRY((dispatch_pair_D<float, S>(a, nd, tod_is_f64 != 0, st, false)));
+    if (tod) CMM_TRY((pair_fwd_stored<float, S>(op, a, nd, tod, tod_is_f64 != 0, st)));
     else if (nc == 1) CMM_TRY((dispatch_pair_T<float, 1, S>(a, nd, 0, st, false)));
     else CMM_TRY((dispatch_pair_T<float, 3, S>(a, nd, 0, st, false)));
   }
@@ -104,6 +191,19 @@ int prepare_pair(cmm_op* op) {
   op->plogC = lc;
   op->pR = 1 << lr;
   op->pC = 1 << lc;
+  if (!op->tod_norm) {
+    const size_t n = (size_t)op->pt->n_det;
+    if (cudaMalloc(&op->tod_norm, (sizeof(double) + 2 * sizeof(float)) * n + sizeof(int) * (1 + (n + 1) / 2)) !=
+        cudaSuccess) {
+      op->tod_norm = nullptr;
+      cudaGetLastError();
+      return fail(CMM_ERR_OOM, "factors of stored data");
+    }
+    op->tod_f = reinterpret_cast<float*>(op->tod_norm + n);
+    op->tod_h = op->tod_f + n;
+    op->tod_list = reinterpret_cast<int*>(op->tod_h + n);
+    CMM_CUDA(cudaMemsetAsync(op->tod_norm, 0, sizeof(double) * n, op->ctx->stream));
+  }
   if (op->prec == CMM_PREC_F64) return prepare_pair64(op);
   if (!op->tw_pair) CMM_TRY(pair_twiddles<float>(op));
   return op->prec == CMM_PREC_BF16 ? prepare_pair_s<float, __nv_bfloat162>(op) : prepare_pair_s<float, float2>(op);

@@ -3,6 +3,11 @@
 // Introduction and Sec. Test setup) for detectors with independent noise: FP32 compute
 // (FP32 or BF16 spectrum storage, tod_pair.cu) and FP64 (tod_pair64.cu).
 //
+// Two detectors in one sequence share its rounding: about 1e-7 of the larger one's values
+// (2^-9 in BF16) reaches the smaller.  Weights and stored data therefore travel in powers
+// of two per detector that make both of order one: w = u w', z = f s, and the filtered
+// data are h y' with h = u / f.  Powers of two change no bit of detectors that are alike.
+//
 // Two detectors d1, d2 share one complex sequence of n_t points, z(t) = s1(t) +
 // i s2(t): each complex element is one time sample of both detectors, so the
 // boresight and rotation tables are read once per element for the two of them, by
@@ -57,13 +62,11 @@
 
 namespace cmm {
 
-// Tuning knobs of this path (compile-time; the defaults are the measured best).
-
 // A binning run in the frame of the scan rotation: for samples of one detector on
 // one pixel, sums of u, u cos 2phi_t and u sin 2phi_t; the detector angle psi_d
 // enters once, when the run is reduced: sum u cos 2(psi + phi) = cos 2psi * sum u
 // cos 2phi - sin 2psi * sum u sin 2phi (and the sine likewise), with the inverse
-// FFT's 1/N folded into (sx, sy) = (cos 2psi, sin 2psi) / N and st = 1/N.
+// FFT's 1/N and the detector's h folded into st = h / N and (sx, sy) = (cos, sin 2psi) st.
 template <typename T>
 struct PairRun {
   int cur = -1;
@@ -118,10 +121,10 @@ __device__ __forceinline__ float2 rot2_of_bore(const int4 b) {
   return make_float2((cf - sf) * (cf + sf) * inv, 2.0f * cf * sf * inv);
 }
 
-// w_d at frequency index kf (0 <= kf <= n_t / 2): the detector's table, else the law
-__device__ __forceinline__ float pair_weight(const TodArgs& a, int d, const float4 cf, int kf) {
-  if (a.wtab) return __ldg(reinterpret_cast<const float*>(a.wtab) + (size_t)d * (a.n_t / 2 + 1) + kf);
-  return filter_weight_law(cf, kf);
+// w_d / u at frequency index kf (0 <= kf <= n_t / 2) from the detector's table (cf.x = 1 / u)
+template <typename T>
+__device__ __forceinline__ T pair_table(const TodArgs& a, int d, const V4<T>& cf, int kf) {
+  return cf.x * __ldg(reinterpret_cast<const T*>(a.wtab) + (size_t)d * (a.n_t / 2 + 1) + kf);
 }
 
 // w of one detector from log2 of its frequency index
@@ -133,8 +136,8 @@ __device__ __forceinline__ float law_weight(const float4 cf, float lk) {
 __device__ __forceinline__ void pair_weights(const TodArgs& a, int d1, int d2, const float4 cf1, const float4 cf2,
                                              bool two, int kf, float& w1, float& w2) {
   if (a.wtab) {
-    w1 = pair_weight(a, d1, cf1, kf);
-    w2 = two ? pair_weight(a, d2, cf2, kf) : 0.f;
+    w1 = pair_table<float>(a, d1, cf1, kf);
+    w2 = two ? pair_table<float>(a, d2, cf2, kf) : 0.f;
   } else {
     const float lk = __log2f(small_int_to_float(kf == 0 ? 1 : kf));
     w1 = law_weight(cf1, lk);
@@ -174,9 +177,8 @@ __device__ __forceinline__ double exp2_tab(double y, const double* __restrict__ 
 __device__ __forceinline__ void pair_ab(const TodArgs& a, int d1, int d2, const double4_32a& cf1, const double4_32a& cf2,
                                         bool two, int kf, double& ha, double& hb) {
   if (a.wtab) {
-    const double* w = reinterpret_cast<const double*>(a.wtab) + kf;
-    const double w1 = __ldg(w + (size_t)d1 * (a.n_t / 2 + 1));
-    const double w2 = two ? __ldg(w + (size_t)d2 * (a.n_t / 2 + 1)) : 0.0;
+    const double w1 = pair_table<double>(a, d1, cf1, kf);
+    const double w2 = two ? pair_table<double>(a, d2, cf2, kf) : 0.0;
     ha = 0.5 * (w1 + w2);
     hb = 0.5 * (w1 - w2);
     return;
@@ -296,33 +298,113 @@ __global__ void __launch_bounds__(PairShape<T, R>::THREADS, PairShape<T, R>::MIN
   pair_fwd_store<T, S, R>(a, x, q, c, i, ad);
 }
 
+// The sum of squares of a thread's values in FP64, by itself, where those of type T leave
+// its range; NaN where a value is not finite.
+template <typename T>
+__device__ __noinline__ void add_squares_far(double* out, const T (&v)[kE]) {
+  T m = 0;
+  bool finite = true;
+  for (int e = 0; e < kE; ++e) {
+    finite = finite && isfinite(v[e]);
+    m = max(m, abs(v[e]));
+  }
+  if (!finite) {
+    atomicAdd(out, (double)NAN);
+  } else if (m > (T)0) {
+    double d = 0.0;
+    for (int e = 0; e < kE; ++e) {
+      const double q = (double)v[e] / (double)m;
+      d += q * q;
+    }
+    const double mm = min(max((double)m, 1e-150), 1e150);   // its square within FP64
+    atomicAdd(out, d * mm * mm);
+  }
+}
+
+// The warp's sums of squares of both numbers of x, in lane 0.
+template <typename T>
+__device__ __forceinline__ V2<T> warp_squares(const V2<T> (&x)[kE], bool on1, bool on2, double* out) {
+  constexpr T lo = sizeof(T) == 4 ? (T)1e-24 : (T)1e-200, hi = sizeof(T) == 4 ? (T)1e30 : (T)1e200;
+  V2<T> s{(T)0, (T)0};
+#pragma unroll
+  for (int e = 0; e < kE; ++e) s = pfma(x[e], x[e], s);
+  const bool far1 = on1 && !(s.x > lo && s.x < hi), far2 = on2 && !(s.y > lo && s.y < hi);   // zero and NaN too
+  if (far1 || far2) {
+    T v[kE];
+    for (int j = 0; j < 2; ++j) {
+      if (!(j ? far2 : far1)) continue;
+#pragma unroll
+      for (int e = 0; e < kE; ++e) v[e] = j ? x[e].y : x[e].x;
+      add_squares_far<T>(out + j, v);
+      (j ? s.y : s.x) = (T)0;
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+    s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+  }
+  return s;
+}
+
 // The same from stored time-ordered data D [n_det][n_t] (the right-hand side): a half-warp
-// reads 16 consecutive samples of either detector.  P^T N^-1 d of 1024 x 2^20 stored FP32
-// samples: 11.1 -> 7.0 ms (the one-detector packing, whose forward pass from stored data
-// is the generic kernel), 128 x 2^18 381 -> 231 us.
-template <typename T, typename S, int R, typename D>
+// reads 16 consecutive samples of either detector, times its factor f; a detector of factor
+// 0 (no weight, or not finite) counts as zero.
+//
+// Data may be as loud as they like (a glitch, a drift, a cut detector), so the noise model's
+// guess of f is checked against the data: the first pass sums their squares on the way,
+// k_tod_gains lists the pairs whose detectors differ, and the LIST form transforms those
+// again with measured factors.  Reading the data for their level before the transform would
+// cost every call a pass over them (537 MB at 256 x 2^19: 80 us).  One FP64 atomic per
+// block and detector, and no load waits for a factor: with one atomic per warp, whose
+// blocks meet on the addresses of a few pairs, and with such waits 935 us a right-hand
+// side of 256 x 2^19, now 840; 825 without the factors, of which 8 us are the two small
+// kernels when no pair is listed, and 1350 in the one-detector packing, whose forward pass
+// from stored data is the generic kernel.
+template <typename T, typename S, int R, typename D, bool LIST>
 __global__ void __launch_bounds__(PairShape<T, R>::THREADS, PairShape<T, R>::MINB) k_pair_fwd_tod(const TodArgs a, int nd) {
   using V = V2<T>;
   constexpr int TPC = R / kE;
   constexpr int J = PairShape<T, R>::J;
   if (a.done && *a.done) return;
   extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ V sums[PairShape<T, R>::THREADS / 32];
   const int cl = threadIdx.x % J;
   const int i = threadIdx.x / J;
   const int c = blockIdx.x * J + cl;
   const ColJ<J, V> ad{reinterpret_cast<V*>(smraw), cl};
-  const int q = blockIdx.y;
-  const bool two = 2 * q + 1 < nd;
-  const D* t1 = reinterpret_cast<const D*>(a.tod) + (size_t)(a.d0 + 2 * q) * a.n_t + c;
-  const D* t2 = two ? t1 + a.n_t : t1;
-  V x[kE];
+  const int nq = LIST ? a.tod_list[0] : (int)gridDim.y;
+  for (int j = blockIdx.y; j < nq; j += gridDim.y) {   // LIST: over the listed pairs, else once
+    const int q = LIST ? a.tod_list[1 + j] : j;
+    const bool two = 2 * q + 1 < nd;
+    const int d1 = a.d0 + 2 * q, d2 = two ? d1 + 1 : d1;
+    const T f1 = (T)a.tod_f[d1], f2 = two ? (T)a.tod_f[d2] : (T)0;
+    const D* t1 = reinterpret_cast<const D*>(a.tod) + (size_t)d1 * a.n_t + c;
+    const D* t2 = reinterpret_cast<const D*>(a.tod) + (size_t)d2 * a.n_t + c;
+    const bool on1 = f1 != (T)0, on2 = f2 != (T)0;   // uniform over the block
+    V x[kE];
 #pragma unroll
-  for (int e = 0; e < kE; ++e) {
-    const int o = (i + e * TPC) * a.C;
-    const T v1 = (T)__ldcs(t1 + o), v2 = (T)__ldcs(t2 + o);
-    x[e] = V{v1, two ? v2 : (T)0};
+    for (int e = 0; e < kE; ++e) {
+      const int o = (i + e * TPC) * a.C;
+      x[e] = pmul(V{f1, f2}, V{(T)__ldcs(t1 + o), (T)__ldcs(t2 + o)});
+    }
+    if (!on1 || !on2) {   // whatever is stored there, NaN too
+#pragma unroll
+      for (int e = 0; e < kE; ++e) x[e] = V{on1 ? x[e].x : (T)0, on2 ? x[e].y : (T)0};
+    }
+    if constexpr (!LIST) {
+      const V s = warp_squares<T>(x, on1, on2, a.tod_norm + d1);
+      if ((threadIdx.x & 31) == 0) sums[threadIdx.x >> 5] = s;
+    }
+    pair_fwd_store<T, S, R>(a, x, q, c, i, ad);   // with barriers between its stages
+    if constexpr (LIST) {
+      __syncthreads();   // the next pair reuses the exchange buffer
+    } else if (threadIdx.x < (two ? 2 : 1)) {
+      double s = 0.0;
+      for (int w = 0; w < PairShape<T, R>::THREADS / 32; ++w) s += widen(threadIdx.x ? sums[w].y : sums[w].x);
+      if (s > 0.0) atomicAdd(a.tod_norm + d1 + threadIdx.x, s);
+    }
   }
-  pair_fwd_store<T, S, R>(a, x, q, c, i, ad);
 }
 
 // ------------------------------------------------------------------ pass F (filter)
@@ -430,13 +512,14 @@ __global__ void __launch_bounds__(PairFilterShape<T, RadProd<RC...>::value, E>::
     const V4<T> cf1 = reinterpret_cast<const V4<T>*>(a.coef)[d1];
     const V4<T> cf2 = reinterpret_cast<const V4<T>*>(a.coef)[d2];
     const int n = (int)a.N;
-    float tv1[kMaxCorrModes], tv2[kMaxCorrModes];   // the detectors' templates
+    float tv1[kMaxCorrModes], tv2[kMaxCorrModes];   // the detectors' templates, as their data times f
     const int slots = pair_corr_slots(a.R, C);
     if constexpr (MODE == kPairMerge) {
+      const float f1 = a.tod_f ? a.tod_f[d1] : 1.f, f2 = a.tod_f ? a.tod_f[d2] : 1.f;
 #pragma unroll
       for (int j = 0; j < kMaxCorrModes; ++j) {
-        tv1[j] = j < a.corr_r ? a.corrV[d1 * a.corr_r + j] : 0.f;
-        tv2[j] = j < a.corr_r ? a.corrV[d2 * a.corr_r + j] : 0.f;
+        tv1[j] = j < a.corr_r ? f1 * a.corrV[d1 * a.corr_r + j] : 0.f;
+        tv2[j] = j < a.corr_r ? f2 * a.corrV[d2 * a.corr_r + j] : 0.f;
       }
     }
 #pragma unroll
@@ -521,8 +604,9 @@ __global__ void __launch_bounds__(kCorrThreads) k_pair_corr(const TodArgs a, int
       const int dd = a.d0 + min(2 * q0 + d, n_det - 1);
       const bool real = 2 * q0 + d < n_det;   // the missing partner of an odd last detector
       coef[d] = reinterpret_cast<const float4*>(a.coef)[dd];
+      const float h = a.tod_h[dd];   // w V S = (w / u) (h V) (f S)
 #pragma unroll
-      for (int j = 0; j < RM; ++j) V[d][j] = real ? a.corrV[dd * RM + j] : 0.f;
+      for (int j = 0; j < RM; ++j) V[d][j] = real ? h * a.corrV[dd * RM + j] : 0.f;
     }
     __syncthreads();
 #pragma unroll 4
@@ -533,10 +617,9 @@ __global__ void __launch_bounds__(kCorrThreads) k_pair_corr(const TodArgs a, int
       if (self) B.y = -B.y;
       float w1, w2;
       if (a.wtab) {
-        const float* w = reinterpret_cast<const float*>(a.wtab) + kf;
         const int d1 = a.d0 + 2 * (q0 + q);
-        w1 = __ldg(w + (size_t)d1 * (a.n_t / 2 + 1));
-        w2 = __ldg(w + (size_t)min(d1 + 1, a.d0 + n_det - 1) * (a.n_t / 2 + 1));
+        w1 = pair_table<float>(a, d1, coef[2 * q], kf);
+        w2 = pair_table<float>(a, min(d1 + 1, a.d0 + n_det - 1), coef[2 * q + 1], kf);
       } else {
         w1 = law_weight(coef[2 * q], lk);
         w2 = law_weight(coef[2 * q + 1], lk);
@@ -620,6 +703,7 @@ __global__ void __launch_bounds__(PairShape<T, R>::THREADS, PairShape<T, R>::MIN
   const V* pol = reinterpret_cast<const V*>(a.pol);
   const V pol1 = pol[d1], pol2 = pol[d2];
   const int2 off1 = a.det_off[d1], off2 = a.det_off[d2];
+  const T st1 = scale * (T)a.tod_h[d1], st2 = scale * (T)a.tod_h[d2];
   int* pst = reinterpret_cast<int*>(smf + R * BS);   // pixels of one pass: [detector][RPP][PS]
   for (int kr0 = 0; kr0 < R; kr0 += RPP) {
     const int kr = kr0 + br;
@@ -698,13 +782,13 @@ __global__ void __launch_bounds__(PairShape<T, R>::THREADS, PairShape<T, R>::MIN
       p[0] = P0.x; p[1] = P0.y; p[2] = P0.z; p[3] = P0.w;
       p[4] = P1.x; p[5] = P1.y; p[6] = P1.z; p[7] = P1.w;
       const V pl = dd ? pol2 : pol1;
-      const T sx = scale * pl.x, sy = scale * pl.y;
+      const T st = dd ? st2 : st1, sx = st * pl.x, sy = st * pl.y;
       PairRun<T> run;
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
         const T u = dd ? yv[k].y : yv[k].x;
         if (p[k] != run.cur) {
-          pair_run_close<NC>(acc, run, npix, scale, sx, sy);
+          pair_run_close<NC>(acc, run, npix, st, sx, sy);
           run.cur = p[k];
           run.t = run.c = run.s = 0;
         }
@@ -714,7 +798,7 @@ __global__ void __launch_bounds__(PairShape<T, R>::THREADS, PairShape<T, R>::MIN
           run.s = fma(r2[k].y, u, run.s);
         }
       }
-      pair_run_close<NC>(acc, run, npix, scale, sx, sy);
+      pair_run_close<NC>(acc, run, npix, st, sx, sy);
     }
     if constexpr (!CACHED) __syncthreads();   // the staging is rewritten by the next pass
   }
@@ -771,25 +855,54 @@ inline int dispatch_pair_T(const TodArgs& a, int nd, int pass, cudaStream_t st, 
 }
 
 // Forward pass from stored data (a.tod).
-template <typename T, typename S, int R>
+// LIST: the pairs of a.tod_list, whose number the device knows; few blocks, since the list
+// is empty for data like their noise model (8 to a column: 3 us at 256 x 2^19).
+template <typename T, typename S, int R, bool LIST>
 inline int run_pair_D(const TodArgs& a, int nd, bool f64, cudaStream_t st, bool attr_only) {
   constexpr int J = PairShape<T, R>::J;
   const int smem = (int)(sizeof(V2<T>) * R * J);
-  const auto k = f64 ? k_pair_fwd_tod<T, S, R, double> : k_pair_fwd_tod<T, S, R, float>;
+  const auto k = f64 ? k_pair_fwd_tod<T, S, R, double, LIST> : k_pair_fwd_tod<T, S, R, float, LIST>;
   if (attr_only) {
     CMM_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     return CMM_OK;
   }
-  k<<<dim3(a.C / J, (nd + 1) / 2), PairShape<T, R>::THREADS, smem, st>>>(a, nd);
+  const int pairs = (nd + 1) / 2;
+  k<<<dim3(a.C / J, LIST ? std::min(pairs, 8) : pairs), PairShape<T, R>::THREADS, smem, st>>>(a, nd);
   CMM_LAUNCH_CHECK();
   return CMM_OK;
 }
 
-template <typename T, typename S>
+template <typename T, typename S, bool LIST>
 inline int dispatch_pair_D(const TodArgs& a, int nd, bool f64, cudaStream_t st, bool attr_only) {
-  if (a.logR == 6) return run_pair_D<T, S, 64>(a, nd, f64, st, attr_only);
-  if (a.logR == 7) return run_pair_D<T, S, 128>(a, nd, f64, st, attr_only);
-  return run_pair_D<T, S, 256>(a, nd, f64, st, attr_only);
+  if (a.logR == 6) return run_pair_D<T, S, 64, LIST>(a, nd, f64, st, attr_only);
+  if (a.logR == 7) return run_pair_D<T, S, 128, LIST>(a, nd, f64, st, attr_only);
+  return run_pair_D<T, S, 256, LIST>(a, nd, f64, st, attr_only);
+}
+
+int launch_tod_gains(const cmm_op* op, const TodArgs& a, int nd, cudaStream_t st);
+
+// The whole forward pass from stored data; leaves the factors in a for the passes after it.
+template <typename T, typename S>
+inline int pair_fwd_stored(const cmm_op* op, TodArgs& a, int nd, const void* tod, bool f64, cudaStream_t st) {
+  a.tod = tod;
+  a.tod_f = op->nz->tod_guess;
+  CMM_TRY((dispatch_pair_D<T, S, false>(a, nd, f64, st, false)));
+  CMM_TRY(launch_tod_gains(op, a, nd, st));
+  a.tod_f = op->tod_f;
+  return dispatch_pair_D<T, S, true>(a, nd, f64, st, false);
+}
+
+// The path's coefficients: those of A, then those of stored data.
+inline const char* pair_coef(const cmm_op* op) {
+  return op->prec == CMM_PREC_F64 ? reinterpret_cast<const char*>(op->nz->pair64)
+                                  : reinterpret_cast<const char*>(op->nz->pair32);
+}
+
+// The factors of stored data in the passes after the forward one.
+inline void stored_gains(const cmm_op* op, TodArgs& a) {
+  a.coef = pair_coef(op) + op->pt->n_det * (op->prec == CMM_PREC_F64 ? sizeof(double4_32a) : sizeof(float4));
+  a.tod_f = op->tod_f;
+  a.tod_h = op->tod_h;
 }
 
 template <typename T, typename S, int MODE, int E, int... RC>
@@ -845,6 +958,7 @@ inline TodArgs pair_args(const cmm_op* op, int d0) {
   a.logC = op->plogC;
   a.tw = op->tw_pair;
   a.twl = tw_layout(op->pR, op->pC);
+  a.coef = pair_coef(op);
   return a;
 }
 
@@ -875,7 +989,10 @@ inline int pair_twiddles(cmm_op* op) {
 template <typename T, typename S>
 inline int prepare_pair_s(cmm_op* op) {
   TodArgs a = pair_args(op, 0);
-  for (const bool f64 : {false, true}) CMM_TRY((dispatch_pair_D<T, S>(a, 0, f64, nullptr, true)));
+  for (const bool f64 : {false, true}) {
+    CMM_TRY((dispatch_pair_D<T, S, false>(a, 0, f64, nullptr, true)));
+    CMM_TRY((dispatch_pair_D<T, S, true>(a, 0, f64, nullptr, true)));
+  }
   if (op->pt->ncomp == 1) CMM_TRY((dispatch_pair_T<T, 1, S>(a, 0, 0, nullptr, true)));
   else CMM_TRY((dispatch_pair_T<T, 3, S>(a, 0, 0, nullptr, true)));
   if constexpr (sizeof(T) == 4) {

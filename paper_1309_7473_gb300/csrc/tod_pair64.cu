@@ -29,12 +29,12 @@ __global__ void k_lg2(long long n, double* __restrict__ out) {
 
 int launch_apply_chunk_pair64(cmm_op* op, int d0, int nd, const void* tod, int tod_is_f64, int pass) {
   TodArgs a = pair_args(op, d0);
-  a.tod = tod;
+  if (tod) stored_gains(op, a);
   cudaStream_t st = op->ctx->stream;
   const bool t_only = op->pt->ncomp == 1;
   if (pass < 0 || pass == 0) {
     TraceRange tr("A: P m + column FFTs (two detectors per sequence, FP64)");
-    if (tod) CMM_TRY((dispatch_pair_D<double, double2>(a, nd, tod_is_f64 != 0, st, false)));
+    if (tod) CMM_TRY((pair_fwd_stored<double, double2>(op, a, nd, tod, tod_is_f64 != 0, st)));
     else if (t_only) CMM_TRY((dispatch_pair_T<double, 1, double2>(a, nd, 0, st, false)));
     else CMM_TRY((dispatch_pair_T<double, 3, double2>(a, nd, 0, st, false)));
   }
