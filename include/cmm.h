@@ -225,7 +225,8 @@ int cmm_op_set_pixel_cache(cmm_op* op, int32_t enable);
  * each bin pair (k, n - k) is filtered as Y(k) = a Z(k) + b conj Z(n - k) with
  * a, b = (w_1 +- w_2) / 2.  The rounding of a sequence is that of its larger member, so
  * weights and stored data travel in powers of two per detector that bring the two to the
- * same size, for stored data from their measured level: a loud detector (a glitch, a
+ * same size (in A where weights are more than four from the median, for stored data from
+ * their measured level): a loud detector (a glitch, a
  * drift, garbage under a weight of zero, which is not looked at) leaves its partner's
  * accuracy as it is, and NaN or Inf stay with their detector unless the noise is
  * correlated.  enable == 0 selects the one-detector packing (even and odd samples as one

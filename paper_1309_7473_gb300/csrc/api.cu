@@ -335,7 +335,10 @@ static float near_pow2(double v) {
 // (the law's mean is within a factor of two of it at the usual slopes).  Two detectors
 // share one complex sequence, so the rounding of the larger reaches the smaller: weights
 // are divided by u before the filter and the filtered data multiplied by it after, and
-// stored data, whose noise has variance 1 / w, by the guess before the transform.
+// stored data, whose noise has variance 1 / w, by the guess before the transform.  In A,
+// whose data are alike for all detectors, only weights beyond a factor of four from the
+// median take a unit: inside it a weight lends its partner's filtered data little rounding,
+// and ordinary operators keep their bits.
 static int noise_units(cmm_noise* nz, const std::vector<double>& w) {
   const size_t n = nz->n_det;
   const size_t at32 = sizeof(double4_32a) * 2 * n, at_unit = at32 + sizeof(float4) * 2 * n;
@@ -346,8 +349,14 @@ static int noise_units(cmm_noise* nz, const std::vector<double>& w) {
   float4* c32 = reinterpret_cast<float4*>(host + at32);
   float* unit = reinterpret_cast<float*>(host + at_unit);
   float* guess = reinterpret_cast<float*>(host + at_guess);
+  std::vector<double> some;
+  for (double v : w)
+    if (v > 0) some.push_back(v);
+  std::nth_element(some.begin(), some.begin() + some.size() / 2, some.end());
+  const double median = some.empty() ? 1.0 : some[some.size() / 2];
   for (size_t d = 0; d < n; ++d) {
-    unit[d] = 1.0f;
+    const double rel = w[d] / median;
+    unit[d] = rel >= 0.25 && rel <= 4.0 ? 1.0f : near_pow2(rel);
     unit[n + d] = near_pow2(w[d]);
     guess[d] = near_pow2(std::sqrt(w[d]));
     for (size_t q = d; q < 2 * n; q += n) {
