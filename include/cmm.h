@@ -441,9 +441,10 @@ int cmm_batch_solve(int32_t n, cmm_op* const* ops, cmm_precon* const* pcs, const
  * applications of A for every candidate: the two-detector packing (where it
  * applies; its split of n_samp is fixed) and every split N = R C of the
  * one-detector packing that the kernels support.  Keeps the fastest and remembers
- * it for operators of the same (n_samp, n_det, precision, ncomp) in this process
- * and, if cache_path is not NULL, in that text file (read first, appended to; the
- * last field is 0 for the two-detector packing, else log2 R).  *chosen_logR (may
+ * it for operators of the same (n_samp, n_det, precision, ncomp, correlated modes) in
+ * this process and, if cache_path is not NULL, in that text file (read first, appended
+ * to; a line is these five and the decision, 0 for the two-detector packing, else
+ * log2 R; lines without the mode count are read where the decision is 0).  *chosen_logR (may
  * be NULL) receives log2 R of the chosen split, *chosen_pair (may be NULL) 1 for
  * the two-detector packing, else 0; *best_ms (may be NULL) the time of one
  * application, or -1 when the decision came from a cache. */

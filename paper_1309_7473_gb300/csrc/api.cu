@@ -1543,12 +1543,25 @@ int cmm_solve_host(cmm_op* op, cmm_precon* pc, const double* b_host, double* x_h
 namespace {
 struct TuneKey {
   int64_t n_t;
-  int n_det, prec, ncomp;
+  int n_det, prec, ncomp, modes;   // modes: of the noise correlated between detectors
   bool operator==(const TuneKey& o) const {
-    return n_t == o.n_t && n_det == o.n_det && prec == o.prec && ncomp == o.ncomp;
+    return n_t == o.n_t && n_det == o.n_det && prec == o.prec && ncomp == o.ncomp && modes == o.modes;
   }
 };
 std::vector<std::pair<TuneKey, int>> g_tune_cache;
+
+// One line of the cache file: the key and the decision.  Lines without the mode count were
+// written by every kind of noise, and for FP64 before it had the two-detector packing:
+// they count where they name that packing, which only independent noise could choose then.
+bool parse_tuned(const char* line, TuneKey& k, int& v) {
+  long long nt;
+  int f[5];
+  const int n = std::sscanf(line, "%lld %d %d %d %d %d", &nt, f, f + 1, f + 2, f + 3, f + 4);
+  if (n != 6 && !(n == 5 && f[3] == 0)) return false;
+  k = TuneKey{nt, f[0], f[1], f[2], n == 6 ? f[3] : 0};
+  v = n == 6 ? f[4] : 0;
+  return true;
+}
 }  // namespace
 
 // Decision values of the tuner (process cache and file): 0 = two-detector packing
@@ -1571,10 +1584,14 @@ int cmm_autotune(cmm_op* op, int32_t reps, const char* cache_path, int32_t* chos
                  double* best_ms) {
   if (!op || reps <= 0) return fail(CMM_ERR_ARG, "bad argument");
   CMM_CUDA(cudaSetDevice(op->ctx->device));
-  const TuneKey key{op->pt->n_t, op->pt->n_det, op->prec, op->pt->ncomp};
+  const TuneKey key{op->pt->n_t, op->pt->n_det, op->prec, op->pt->ncomp, op->nz->corr_r};
   const int logN = op->logR + op->logC;
-  const bool pair_ok = pair_path_fits(op) && op->nz->corr_r == 0;
-  auto valid = [&](int v) { return (v == 0 && pair_ok) || (v > 0 && v < logN); };
+  const bool pair_ok = pair_path_fits(op);
+  const int lr0 = op->logR;
+  // Correlated noise is served in the two-detector packing and in the fast kernels' own
+  // split (where the operator cannot serve it, the application that needs it fails).
+  const bool corr = op->nz->corr_r > 0 && fast_path_ok(op) && op->chunk >= op->pt->n_det;
+  auto valid = [&](int v) { return (v == 0 && pair_ok) || (v > 0 && v < logN && (!corr || v == lr0)); };
   // cached decision (process-wide, then the optional file)
   for (auto& e : g_tune_cache)
     if (e.first == key && valid(e.second)) {
@@ -1585,10 +1602,11 @@ int cmm_autotune(cmm_op* op, int32_t reps, const char* cache_path, int32_t* chos
     }
   if (cache_path) {
     if (FILE* f = std::fopen(cache_path, "r")) {
-      long long nt;
-      int nd, pr, nc, v;
-      while (std::fscanf(f, "%lld %d %d %d %d", &nt, &nd, &pr, &nc, &v) == 5)
-        if (TuneKey{nt, nd, pr, nc} == key && valid(v)) {
+      char line[256];
+      TuneKey k;
+      int v;
+      while (std::fgets(line, sizeof(line), f))
+        if (parse_tuned(line, k, v) && k == key && valid(v)) {
           std::fclose(f);
           g_tune_cache.push_back({key, v});
           CMM_TRY(apply_decision(op, v));
@@ -1604,7 +1622,7 @@ int cmm_autotune(cmm_op* op, int32_t reps, const char* cache_path, int32_t* chos
   std::vector<int> cand;
   if (pair_ok) cand.push_back(0);
   for (int lr = 6; lr <= 8; ++lr)
-    if (logN - lr >= 6 && logN - lr <= 12 && op->prec != CMM_PREC_F64) cand.push_back(lr);
+    if (logN - lr >= 6 && logN - lr <= 12 && op->prec != CMM_PREC_F64 && (!corr || lr == lr0)) cand.push_back(lr);
   if (cand.empty() || op->prec == CMM_PREC_F64) cand.push_back(op->logR);   // the generic kernels
   const size_t bytes = sizeof(double) * op->pt->ncomp * op->pt->npix;
   CMM_CUDA(cudaMemsetAsync(op->tmp_a, 0, bytes, op->ctx->stream));
@@ -1616,6 +1634,7 @@ int cmm_autotune(cmm_op* op, int32_t reps, const char* cache_path, int32_t* chos
   int s = CMM_OK;
   for (int v : cand) {
     s = apply_decision(op, v);
+    if (s == CMM_OK && corr) s = op_sync_corr(op);   // its tables in this packing's order
     if (s != CMM_OK) break;
     s = apply_A_dev(op, op->tmp_a, op->tmp_b);   // warm-up
     if (s != CMM_OK) break;
@@ -1633,12 +1652,17 @@ int cmm_autotune(cmm_op* op, int32_t reps, const char* cache_path, int32_t* chos
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
+  // the timed splits are not left behind: what else the operator does needs its own
+  if (op->logR != lr0) {
+    const int s2 = op_set_split(op, lr0);
+    if (s == CMM_OK) s = s2;
+  }
   if (s != CMM_OK) return s;
   CMM_TRY(apply_decision(op, best));
   g_tune_cache.push_back({key, best});
   if (cache_path) {
     if (FILE* f = std::fopen(cache_path, "a")) {
-      std::fprintf(f, "%lld %d %d %d %d\n", (long long)key.n_t, key.n_det, key.prec, key.ncomp, best);
+      std::fprintf(f, "%lld %d %d %d %d %d\n", (long long)key.n_t, key.n_det, key.prec, key.ncomp, key.modes, best);
       std::fclose(f);
     }
   }
