@@ -351,9 +351,8 @@ def run_ours(args, rank, world):
             op.set_pair_packing(False)
             prof_single = cmm.cmm_profile_apply(op.h, b, mo, 3)
             op.set_pair_packing(True)
-    fast = args.prec != "f64" and (1 << 13) <= scan.n_t <= (1 << 20)   # the register-FFT kernels
-    # two detectors per complex FFT unless the noise is correlated between detectors
-    pre = ("k_pair_" if args.corr_modes == 0 else "k_fast_") if fast else "k_tod_"
+    path = apply_path(args.prec, scan.n_t, args.corr_modes)
+    pre = path["kernels"]
     names = [pre + "fwd (pointing + gather + column FFTs)", pre + "filter (row FFTs + N^-1)",
              pre + "inv_bin (inverse column FFTs + P^T)"]
     chunk_dets = min(op_chunk(op, scan, args), scan.n_det)
@@ -438,7 +437,7 @@ def run_ours(args, rank, world):
                   ("cached_pointing_ms_per_pass" if args.pointing != "cached" else "on_the_fly_ms_per_pass"):
                       None if prof_other is None else {"fwd": prof_other[0], "filter": prof_other[1],
                                                        "inv_bin": prof_other[2]},
-                  "packing": "two detectors per complex FFT" if prof_single is not None else "one detector",
+                  "packing": "two detectors per complex FFT" if pre == "k_pair_" else "one detector",
                   "one_detector_packing_ms": None if prof_single is None else prof_single[4],
                   "one_detector_packing_ms_per_pass": None if prof_single is None else {
                       "fwd": prof_single[0], "filter": prof_single[1], "inv_bin": prof_single[2]}},
@@ -456,10 +455,9 @@ def run_ours(args, rank, world):
         "setup_seconds": round(setup_s, 2),
         "clocks": clocks,
     }
-    # the FP32 two-detector path: the application's last flush writes the map
-    map_out = 0 if args.prec != "f64" and args.corr_modes == 0 else 1
-    out["gpu_launches"] = (launches_per_iteration(scan.n_det, chunk_dets, CIRC_FUSED_LAUNCHES, map_out, CG_FUSED_LAUNCHES) * args.steps
-                           + SETUP_LAUNCHES + CIRC_FUSED_LAUNCHES)
+    per_step = launches_per_iteration(scan.n_det, chunk_dets, CIRC_FUSED_LAUNCHES, path["map_out"], CG_FUSED_LAUNCHES,
+                                      path["filter"], path["flush"])
+    out["gpu_launches"] = per_step * args.steps + SETUP_LAUNCHES + CIRC_FUSED_LAUNCHES
     return out
 
 
@@ -655,10 +653,23 @@ def cufft_filter_ms(scan, noise, dev, stream):
                     "excludes P and P^T", "ms": ms}
 
 
-def launches_per_iteration(n_det, chunk, circ=None, map_out=1, cg=None):
+def apply_path(prec, n_t, corr_modes):
+    """The kernels of an A-application: two detectors per complex FFT at 2^13 to 2^20
+    samples in every precision, else the generic ones.  The last FP32 flush writes the
+    map itself; FP64 bins straight into the accumulator, which one kernel copies out.
+    Correlated noise cuts the filter pass into the forward rows, the cross-detector step
+    and the merge with the inverse rows."""
+    pair = (1 << 13) <= n_t <= (1 << 20)
+    flush = pair and prec != "f64"
+    return {"kernels": "k_pair_" if pair else "k_tod_", "flush": flush, "map_out": 0 if flush else 1,
+            "filter": 3 if corr_modes > 0 else 1}
+
+
+def launches_per_iteration(n_det, chunk, circ=None, map_out=1, cg=None, filter_launches=1, flush=True):
     """Kernels of one circulant-PCG iteration: the A-application (map copy in, per
-    chunk one forward and one filter launch and, per 2048 detectors (eight FP32
-    partial maps of 256 detectors), one inverse + binning launch and one flush; a map
+    chunk one forward launch, the filter's and, per 2048 detectors (eight FP32
+    partial maps of 256 detectors), one inverse + binning launch and one flush, or one
+    inverse + binning launch where nothing is flushed; a map
     copy out where the flush does not write the map), the `cg` update kernels (by
     default those of the flexible solves) and the circulant preconditioner: `circ`
     kernels, by default those of the maps that the line FFTs serve (Sigma^-1,
@@ -667,7 +678,7 @@ def launches_per_iteration(n_det, chunk, circ=None, map_out=1, cg=None):
     maps = min(8, max(1, math.ceil(chunk / 256)))
     for d0 in range(0, n_det, chunk):
         nd = min(chunk, n_det - d0)
-        a += 2 + 2 * math.ceil(nd / (256 * maps))
+        a += 1 + filter_launches + (2 * math.ceil(nd / (256 * maps)) if flush else 1)
     return a + (CG_LAUNCHES if cg is None else cg) + (CIRC_LAUNCHES if circ is None else circ)
 
 
