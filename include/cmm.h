@@ -204,7 +204,8 @@ int cmm_noise_diag(cmm_noise* nz, double* diag_host);
  * 32 <= n_samp <= 2^22.  det_chunk > 0 bounds how many detectors share one pass
  * through the intermediate spectrum buffer (<= 0: automatic).  The handle owns
  * that buffer (n_chunk, rounded up to even, * n_samp * 4 bytes in F32, 8 in F64,
- * 2 in BF16) and a few map-sized buffers.
+ * 2 in BF16), a few map-sized buffers and, in F64 at 2^13 to 2^20 samples, tables of
+ * 20 bytes a sample of one detector.
  */
 int cmm_op_create(cmm_ctx* ctx, cmm_pointing* pt, cmm_noise* nz, int32_t precision,
                   int32_t det_chunk, cmm_op** out);

@@ -16,12 +16,13 @@
 // The transforms are mixed-radix Stockham passes in place: every thread takes one
 // butterfly of up to 12 points into registers, so most sides up to a thousand take three
 // passes (900 = 9 10 10, 1200 = 12 10 10), the first reading global memory and the last
-// writing it.  Against one kernel per step (seven, with
-// double-buffered passes of radix 2 to 5, five for 900 and 1200) the planes cross L2
-// four times instead of ten: one apply at 1200 x 900 FP32 154 -> 66 us (rows 17, columns
-// 24, rows 19; 117 MB of maps and blocks: 17 us of HBM), 600 x 450 33 us, 256 x 256 54 -> 26,
-// 64 x 64 35 -> 23 (FP64 59 -> 42).  What bounds it now is latency at 24 warps per SM, and
-// in the last kernel the FP64 pipe (z and its product with r).
+// writing it.  Against one kernel per step (seven, with double-buffered passes of radix 2
+// to 5, five for 900 and 1200) the planes cross L2
+// four times instead of ten.  One apply after another on one stream, FP32: 1200 x 900 155 ->
+// 69 us (rows 19, columns 26, rows 22; 117 MB of maps and blocks: 17 us of HBM), 600 x 450
+// 77 -> 34, 256 x 256 51 -> 25, 64 x 64 35 -> 23 (FP64 58 -> 42); three maps at 1200 x 900 on
+// three streams 130 -> 50 us an apply.  What bounds it now is latency at 24 warps per SM,
+// and in the last kernel the FP64 pipe (z and its product with r).
 #include <math.h>
 
 #include <algorithm>
@@ -159,10 +160,10 @@ __device__ __forceinline__ void cx_dft_n(Cx2<T>* x) {
 
 // Launch shapes.  FP32: at most 12 points a thread (48 registers of data), two columns
 // beside each other to make whole 32-byte sectors, and registers for three row blocks and
-// two column blocks per SM (two and one: 84 against 62 us an apply at 1200 x 900, four row
-// blocks 64, with twiddles formed in registers).  FP64: at most 6 points, since its pipe takes as long for a warp with few
-// lanes as for a full one, so small maps want many threads a line (64 x 64: 45 us an apply
-// in radix 4, 76 in radix 8).
+// two column blocks per SM (two and one: 1.35 times the time of an apply at 1200 x 900, four
+// row blocks 1.03 times, both with twiddles formed in registers).  FP64: at most 6 points,
+// since its pipe takes as long for a warp with few lanes as for a full one, so small maps
+// want many threads a line (64 x 64: 45 us an apply in radix 4, 76 in radix 8).
 template <typename T> struct CircKernel {
   static constexpr int kMaxRad = sizeof(T) == 4 ? 12 : 6;
   static constexpr int kRowThreads = sizeof(T) == 4 ? 256 : 512, kRowBlocks = sizeof(T) == 4 ? 3 : 1;
@@ -184,8 +185,8 @@ __device__ __forceinline__ void butterfly_in(Cx2<T> (&x)[CircKernel<T>::kMaxRad]
     for (int m = 0; m < R; ++m) x[m] = load(i + m * nbf);
   }
   if (twiddle) {
-    // w^m from the table: powers formed in registers lose digits (an apply at 1200 x 900 is 62
-    // us with them instead of 66, but 3e-7 from the line FFTs instead of 1.5e-7)
+    // w^m from the table: powers formed in registers lose digits (an apply at 1200 x 900 is 6 %
+    // faster with them, but 3e-7 from the line FFTs instead of 1.5e-7)
 #pragma unroll
     for (int m = 1; m < R; ++m) {
       const V2<T> w = __ldg(tw + m * step);
@@ -448,7 +449,7 @@ CircPlan circ_plan(int ny, int nx) {
   p.J = CircKernel<T>::kCols;
   if (ny >= 65536 || nx >= 65536 || !plan_line<T>(nx, p.x) || !plan_line<T>(ny, p.y)) return p;
   // whole warps, and more than one row a block only while two blocks per SM are left
-  const int fill = std::max((32 + p.x.width - 1) / p.x.width, (ny + 303) / 304);
+  const int fill = std::max((32 + p.x.width - 1) / p.x.width, (ny + 2 * kSMs - 1) / (2 * kSMs));
   p.rows = std::max(1, std::min(fill, 256 / p.x.width));
   // one column a block where two (375 = 5 5 5 3: 125 threads a line) do not fit
   const auto cols_fit = [&] {

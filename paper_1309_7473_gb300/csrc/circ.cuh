@@ -24,9 +24,12 @@ struct CircPlan {
   int64_t modes() const { return (int64_t)((nx / 2 + J) / J) * J * ny; }   // stored mode blocks
 };
 
-// ok = false where a block cannot hold the lines: more threads a line than the launch
-// bounds (FP32 columns past about 1000 pixels of small factors, FP64 past about 1500) or
-// more than 200 KB of shared memory.  The line FFTs of map.cu serve those sides.
+// ok = false where a block cannot hold the lines: a line takes L / (its smallest radix)
+// threads, of which a row may have 256 (FP64 512) and a column and its mirror together 448
+// (FP64 512), or more than 200 KB of shared memory.  In FP32 (radices to 12) every side of
+// 2, 3 and 5 below 675 and most up to 1200 fit; columns of 675 = 9 5 5 3 and 1024 = 8 8 4 4
+// do not.  In FP64 (radices to 6) one small radix costs more: columns of 640, 800, 810, 960,
+// 972, 1000, 1125, 1152 and 1200 do not fit.  The line FFTs of map.cu serve those sides.
 template <typename T> CircPlan circ_plan(int ny, int nx);
 // Opts the kernels into the plan's shared memory (before any stream capture).
 template <typename T> int circ_prepare(const CircPlan& p);

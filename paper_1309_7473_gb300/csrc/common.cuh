@@ -219,6 +219,7 @@ struct cmm_op {
 
 namespace cmm {
 
+constexpr int kSMs = 152;          // of a GB300: the unit of the grids that are cut to fill it
 constexpr int kRedBlocks = 1024;   // fixed grid of the deterministic reductions
 constexpr int kMaxCorrModes = 4;   // correlated noise modes
 

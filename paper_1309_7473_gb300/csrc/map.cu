@@ -357,8 +357,9 @@ __global__ void k_update_p(double* __restrict__ p, const double* __restrict__ z,
 // and one thread for the divisions, since the FP64 pipe takes 16 cycles an instruction), so
 // no single-block kernel stands between the vector kernels.  With p^T q formed by the
 // application's last kernel an iteration is 10 kernels instead of 15: 20 circulant
-// iterations at 128 x 2^18 on 256 x 256 6.70 -> 6.1 ms; the two kernels take 7 us each at
-// 64 x 64, where the five and the dot product took 22.
+// iterations at 128 x 2^18 on 256 x 256 6.70 -> 6.39 ms; the two kernels take 7 us each at
+// 64 x 64, where the five and the dot product took 22.  FP32-vector solves run them too,
+// with a dot product of their own for p^T q.
 // What a kernel's blocks read, that kernel's block 0 does not write: rho is read by
 // k_cg_dir and written by k_cg_step, rho_new the other way round, and iter is read by
 // k_cg_dir and counted by k_cg_step.  `done` is the exception: block 0 may set it while
@@ -1261,7 +1262,7 @@ int launch_update_p(double* p, const double* z, int64_t n, const SolverDev* st, 
 
 // Two blocks per SM while the partial sums that every block forms weigh, four for maps of
 // more than a million values.
-static int cg_blocks(int64_t n) { return n > (1 << 20) ? 608 : 304; }
+static int cg_blocks(int64_t n) { return (n > (1 << 20) ? 4 : 2) * kSMs; }
 
 int launch_cg_step(SolverDev* st, const double* pq_part, double* x, double* r, const double* p, const double* q, int64_t n,
                    double* rr_part, double* anorm, cudaStream_t s) {

@@ -1,7 +1,7 @@
 // Kernels of the pair-packed path of A = P^T N^-1 P (Eq. 2; pointing of Eq. 1 with the response
 // of Sec. Test setup; N^-1 the per-detector Fourier-diagonal noise filter of the
-// Introduction and Sec. Test setup) for detectors with independent noise: FP32 compute
-// (FP32 or BF16 spectrum storage, tod_pair.cu) and FP64 (tod_pair64.cu).
+// Introduction and Sec. Test setup): FP32 compute (FP32 or BF16 spectrum storage, with or
+// without noise correlated between detectors, tod_pair.cu) and FP64 (tod_pair64.cu).
 //
 // Two detectors in one sequence share its rounding: about 1e-7 of the larger one's values
 // (2^-9 in BF16) reaches the smaller.  Weights and stored data therefore travel in powers

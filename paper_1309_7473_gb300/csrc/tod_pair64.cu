@@ -51,7 +51,7 @@ int launch_apply_chunk_pair64(cmm_op* op, int d0, int nd, const void* tod, int t
 }
 
 // The FP64 tables: twiddles, (cos 2phi, sin 2phi) per sample and log2 per frequency
-// index (24 bytes a sample of one detector, kept by the operator).
+// index (20 bytes a sample of one detector, kept by the operator).
 int prepare_pair64(cmm_op* op) {
   const long long n_t = op->pt->n_t;
   cudaStream_t st = op->ctx->stream;
