@@ -354,13 +354,14 @@ static int noise_units(cmm_noise* nz, const std::vector<double>& w) {
     if (v > 0) some.push_back(v);
   std::nth_element(some.begin(), some.begin() + some.size() / 2, some.end());
   const double median = some.empty() ? 1.0 : some[some.size() / 2];
+  const float per = 1.0f / (float)nz->n_t;   // exact where the path applies
   for (size_t d = 0; d < n; ++d) {
     const double rel = w[d] / median;
-    unit[d] = rel >= 0.25 && rel <= 4.0 ? 1.0f : near_pow2(rel);
-    unit[n + d] = near_pow2(w[d]);
     guess[d] = near_pow2(std::sqrt(w[d]));
     for (size_t q = d; q < 2 * n; q += n) {
-      const float iu = unit[q] > 0 ? 1.0f / unit[q] : 0.0f;
+      const float u = q >= n ? near_pow2(w[d]) : rel >= 0.25 && rel <= 4.0 ? 1.0f : near_pow2(rel);
+      const float iu = u > 0 ? 1.0f / u : 0.0f;
+      unit[q] = u * per;
       const double4_32a c = nz->coef_host[d];
       c64[q] = double4_32a{nz->wtab64 ? (double)iu : c.x * iu, c.y, c.z, c.w};
       c32[q] = float4{nz->wtab64 ? iu : (float)c.x * iu, (float)c.y, (float)c.z, (float)c.w};

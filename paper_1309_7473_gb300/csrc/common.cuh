@@ -157,8 +157,8 @@ struct cmm_noise {
   double* white = nullptr;     // [n_det] 1 / sigma^2, the white level of the law
   std::vector<double> diag_host;
   // two-detector path (noise_units, api.cu), [2][n_det] each, for A and for the right-hand
-  // side: the unit u of the weights (a power of two; 0 without weight) and the coefficients
-  // with 1 / sigma^2 in that unit (with a table: 1 / u, its factor)
+  // side: the unit u of the weights (a power of two; 0 without weight) over n_t, and the
+  // coefficients with 1 / sigma^2 in that unit (with a table: 1 / u, its factor)
   // (one allocation, at pair64)
   double4_32a* pair64 = nullptr;
   float4* pair32 = nullptr;

@@ -101,7 +101,8 @@ struct TodArgs {
   const float* corrV;   // [n_det][corr_r]
   const float* corr_minv;   // [N + 1][r][r] slot order
   float2* corr_s;       // [N][r]
-  // two-detector path, per detector: factor on the data (nullptr: 1) and on the filtered data
+  // two-detector path, per detector: factor on the data (nullptr: 1) and on the filtered
+  // data, the latter with the inverse transform's 1 / n_t
   const float* tod_f;
   const float* tod_h;
   double* tod_norm;     // sums of squares of stored data, times tod_f^2

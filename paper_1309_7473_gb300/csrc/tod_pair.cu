@@ -31,7 +31,8 @@ int launch_flush_maps(const TodArgs& a, int nc, int maps, cudaStream_t st);
 
 // ------------------------------------------------------------------ factors of stored data
 // One block after the first forward pass: from every detector's sum of squares (cleared for
-// the next call) its factors f and h = u / f, and the list of pairs to transform again.
+// the next call) its factors f and h = u / (n_t f), and the list of pairs to transform again.
+// unit: u / n_t.
 //
 // level = mean square of f s.  A pair whose rms differ by less than kTodBalance keeps the
 // guesses: its quieter detector then carries at most about kTodBalance times its own
@@ -94,7 +95,7 @@ __global__ void __launch_bounds__(kGainThreads) k_tod_gains(double* norm, const 
       again = true;
       for (int j = 0; j < 2; ++j) {
         const int d = d0 + 2 * q + j;
-        // the guess over sqrt(level), within 2^+-100, and u / f within FP32
+        // the guess over sqrt(level), within 2^+-100, and h within FP32
         const int eu = ilogbf(unit[d]);
         const int ef = (int)fmin(100.0, fmax(-100.0, ilogbf(guess[d]) - rint(0.5 * log2(level[j]))));
         f[d] = scalbnf(1.0f, min(max(ef, eu - 126), eu + 126));

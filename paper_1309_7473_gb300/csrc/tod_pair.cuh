@@ -6,7 +6,8 @@
 // Two detectors in one sequence share its rounding: about 1e-7 of the larger one's values
 // (2^-9 in BF16) reaches the smaller.  Weights and stored data therefore travel in powers
 // of two per detector that make both of order one: w = u w', z = f s, and the filtered
-// data are h y' with h = u / f.  Powers of two change no bit of detectors that are alike.
+// data are h y' with h = u / f (kept with the inverse transform's 1 / n_t).  Powers of two
+// change no bit of detectors that are alike.
 //
 // Two detectors d1, d2 share one complex sequence of n_t points, z(t) = s1(t) +
 // i s2(t): each complex element is one time sample of both detectors, so the
@@ -66,7 +67,7 @@ namespace cmm {
 // one pixel, sums of u, u cos 2phi_t and u sin 2phi_t; the detector angle psi_d
 // enters once, when the run is reduced: sum u cos 2(psi + phi) = cos 2psi * sum u
 // cos 2phi - sin 2psi * sum u sin 2phi (and the sine likewise), with the inverse
-// FFT's 1/N and the detector's h folded into st = h / N and (sx, sy) = (cos, sin 2psi) st.
+// FFT's 1/N and the detector's u / f in st = h and (sx, sy) = (cos, sin 2psi) st.
 template <typename T>
 struct PairRun {
   int cur = -1;
@@ -604,7 +605,7 @@ __global__ void __launch_bounds__(kCorrThreads) k_pair_corr(const TodArgs a, int
       const int dd = a.d0 + min(2 * q0 + d, n_det - 1);
       const bool real = 2 * q0 + d < n_det;   // the missing partner of an odd last detector
       coef[d] = reinterpret_cast<const float4*>(a.coef)[dd];
-      const float h = a.tod_h[dd];   // w V S = (w / u) (h V) (f S)
+      const float h = (float)a.n_t * a.tod_h[dd];   // w V S = (w / u) (u / f V) (f S)
 #pragma unroll
       for (int j = 0; j < RM; ++j) V[d][j] = real ? h * a.corrV[dd * RM + j] : 0.f;
     }
@@ -683,7 +684,6 @@ __global__ void __launch_bounds__(PairShape<T, R>::THREADS, PairShape<T, R>::MIN
   T* acc;
   if constexpr (sizeof(T) == 4) acc = a.acc32 + (long long)((2 * q) / a.flush_dets) * a.acc32_map;
   else acc = a.acc;
-  const T scale = (T)1 / (T)a.N;
   const int npix = (int)a.npix;
   const S* Y = reinterpret_cast<const S*>(a.spec) + (size_t)q * a.N + c + i * a.C;
   V x[kE];
@@ -703,7 +703,6 @@ __global__ void __launch_bounds__(PairShape<T, R>::THREADS, PairShape<T, R>::MIN
   const V* pol = reinterpret_cast<const V*>(a.pol);
   const V pol1 = pol[d1], pol2 = pol[d2];
   const int2 off1 = a.det_off[d1], off2 = a.det_off[d2];
-  const T st1 = scale * (T)a.tod_h[d1], st2 = scale * (T)a.tod_h[d2];
   int* pst = reinterpret_cast<int*>(smf + R * BS);   // pixels of one pass: [detector][RPP][PS]
   for (int kr0 = 0; kr0 < R; kr0 += RPP) {
     const int kr = kr0 + br;
@@ -782,7 +781,8 @@ __global__ void __launch_bounds__(PairShape<T, R>::THREADS, PairShape<T, R>::MIN
       p[0] = P0.x; p[1] = P0.y; p[2] = P0.z; p[3] = P0.w;
       p[4] = P1.x; p[5] = P1.y; p[6] = P1.z; p[7] = P1.w;
       const V pl = dd ? pol2 : pol1;
-      const T st = dd ? st2 : st1, sx = st * pl.x, sy = st * pl.y;
+      // loaded here: held in registers through the pass they cost it 1.3 % (301 x 2^19)
+      const T st = (T)__ldg(a.tod_h + (dd ? d2 : d1)), sx = st * pl.x, sy = st * pl.y;
       PairRun<T> run;
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
